@@ -8,13 +8,13 @@
 // Every convolution runs as an implicit GEMM on the tensor cores (tcgen05, M = 128
 // positions, K = 16 input channels per tap, accumulators in TMEM). All activations are
 // bfloat16 with 16 channels (the 5 gas fields are padded with zeros), so every layer is the
-// same 16 -> 16 kernel with zero-padded weights. Activations are stored line-half-major
-// ([z][y][2][x][8]): each 8-channel half of a line is a contiguous run of 16-byte positions,
-// the row layout of the no-swizzle K-major operand, so an input plane reaches shared memory
-// as bulk copies. One padding column on each side of every staged line (pitch P = n + 2)
-// makes the operand of an in-plane shift (dy, dx) the same tile moved by (dy P + dx) rows:
-// descriptors only, no gather; positions that fall on a padding column give discarded
-// results. The three dz taps of one (dy, dx) form one N = 48 operand that updates three
+// same 16 -> 16 kernel with zero-padded weights. Activations are stored half-major within
+// a plane ([z][2][y][P][8], P = n + 2): each 8-channel half of a line is a contiguous run of
+// 16-byte positions, the row layout of the no-swizzle K-major operand, with the two periodic
+// padding positions stored beside it, so a run of lines of one half is one contiguous piece
+// and reaches shared memory as one bulk copy. The padding makes the operand of an in-plane
+// shift (dy, dx) the same tile moved by (dy P + dx) rows: descriptors only, no gather;
+// positions that fall on a padding column give discarded results. The three dz taps of one (dy, dx) form one N = 48 operand that updates three
 // output planes at once (see the geometry section).
 //
 // Backward: the gradient with respect to a layer's input is the same convolution with the
@@ -184,15 +184,17 @@ __device__ __forceinline__ int wrapi(int i, int n) {
   return i;
 }
 
-// Activations are bfloat16 [B][z][y][2][x][8]: every line holds its 8-channel halves one
-// after the other, each half a contiguous run of 16-byte positions, the row layout of the
-// convolution's shared-memory operand (so a line half arrives with one bulk copy).
-// Element offset of position x, half h of line `line` = (b n + z) n + y:
-__device__ __forceinline__ size_t act_off(long long line, int n, int h, int x) {
-  return ((size_t)(line * 2 + h) * n + x) * 8;
+// Activations are bfloat16 [B][z][2][y][P][8] with P = n + 2: the 8-channel halves of a plane
+// one after the other, each line of a half a contiguous run of 16-byte positions -1 .. n (the
+// first and last repeat x = n - 1 and x = 0), so a run of lines arrives with one bulk copy.
+// Element offset of position x, half h of line y of plane zb = b n + z:
+__device__ __forceinline__ size_t act_off(int zb, int y, int n, int h, int x) {
+  return ((size_t)((zb * 2 + h) * n + y) * (n + 2) + (x + 1)) * 8;
 }
+// elements of one activation array of B instances
+static size_t act_count(int n, int B) { return (size_t)B * n * n * (n + 2) * CH; }
 
-__device__ __forceinline__ void act_store(bf16* base, long long line, int n, int x,
+__device__ __forceinline__ void act_store(bf16* base, int zb, int y, int n, int x,
                                           const float v[16]) {
   uint32_t w[8];
 #pragma unroll
@@ -200,8 +202,20 @@ __device__ __forceinline__ void act_store(bf16* base, long long line, int n, int
     const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
     w[j] = *reinterpret_cast<const uint32_t*>(&p);
   }
-  *reinterpret_cast<uint4*>(base + act_off(line, n, 0, x)) = make_uint4(w[0], w[1], w[2], w[3]);
-  *reinterpret_cast<uint4*>(base + act_off(line, n, 1, x)) = make_uint4(w[4], w[5], w[6], w[7]);
+  uint4* d0 = reinterpret_cast<uint4*>(base + act_off(zb, y, n, 0, x));
+  uint4* d1 = reinterpret_cast<uint4*>(base + act_off(zb, y, n, 1, x));
+  const uint4 q0 = make_uint4(w[0], w[1], w[2], w[3]), q1 = make_uint4(w[4], w[5], w[6], w[7]);
+  *d0 = q0;
+  *d1 = q1;
+  // the periodic padding positions of the line
+  if (x == 0) {
+    d0[n] = q0;
+    d1[n] = q1;
+  }
+  if (x == n - 1) {
+    d0[-n] = q0;
+    d1[-n] = q1;
+  }
 }
 
 struct F5 {
@@ -212,7 +226,7 @@ struct F5 {
 enum { CONV_HIDDEN = 0, CONV_OUT_Y = 1, CONV_OUT_APPLY = 2, CONV_BWD = 3 };
 
 struct ConvArgs {
-  const bf16* in;      // activations [B][n][n][2][n][8]
+  const bf16* in;      // activations [B][n][2][n][n + 2][8]
   const bf16* w;       // packed [27][2][16 rows][8]: row = output channel, K = input channel
   const float* bias;   // [16] (forward) or NULL
   int n, P, L, T, tpl, contig, Zc, R, ring, slot_pos, ncols;
@@ -231,9 +245,8 @@ struct ConvArgs {
 constexpr unsigned long long kDrainNs = 4000000000ull;
 
 // Bulk copies (async proxy, completion counted in bytes on the plane's mbarrier) of input
-// plane gz (periodic) into ring slot `slot_addr`: for each of the L + 2 lines and each
-// 8-channel half, the n interior positions (one copy) and the two periodic padding
-// positions (16 bytes each). Lane k of the issuing warp copies line half k, k + 32, ...
+// plane gz (periodic) into ring slot `slot_addr`: lane h copies the L + 2 padded lines of
+// 8-channel half h, contiguous in memory but for the periodic wrap in y.
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes,
                                          uint64_t* mbar) {
   asm volatile(
@@ -246,20 +259,28 @@ __device__ __forceinline__ uint32_t plane_tx_bytes(const ConvArgs& a) {
   return (uint32_t)(a.L + 2) * 2u * (uint32_t)(a.n + 2) * 16u;
 }
 
+// Lines y, y + 1, ... (periodic), `lines` of them, of half h of plane zb into dst (pitch
+// (n + 2) positions): one copy per piece between wraps.
+__device__ __forceinline__ void fetch_lines(const bf16* in, int zb, int h, int y, int lines, int n,
+                                            uint32_t dst, uint64_t* mbar) {
+  const uint32_t pitch = (uint32_t)(n + 2) * 16u;
+  y = wrapi(y, n);
+  while (lines > 0) {
+    const int c = min(lines, n - y);
+    bulk_g2s(dst, in + act_off(zb, y, n, h, -1), (uint32_t)c * pitch, mbar);
+    dst += (uint32_t)c * pitch;
+    lines -= c;
+    y = 0;
+  }
+}
+
 __device__ __forceinline__ void conv_fetch_plane(const ConvArgs& a, const bf16* in, uint32_t slot_addr,
                                                  int gz, int y0, int lane, uint64_t* mbar) {
-  const int n = a.n, P = a.P, L = a.L;
-  const uint32_t plane_bytes = (uint32_t)a.slot_pos * 16u;
+  const int n = a.n;
   gz = gz < 0 ? gz + n : (gz >= n ? gz - n : gz);
-  for (int k = lane; k < 2 * (L + 2); k += 32) {
-    const int ly = k >> 1, h = k & 1;
-    const int gy = wrapi(y0 - 1 + ly, n);
-    const bf16* src = in + act_off((long long)gz * n + gy, n, h, 0);
-    const uint32_t d = slot_addr + (uint32_t)h * plane_bytes + (uint32_t)(SLK_BEFORE + ly * P) * 16u;
-    bulk_g2s(d + 16u, src, (uint32_t)n * 16u, mbar);                    // x = 0 .. n - 1
-    bulk_g2s(d, src + (size_t)(n - 1) * 8, 16u, mbar);                  // x = -1 -> n - 1
-    bulk_g2s(d + (uint32_t)(n + 1) * 16u, src, 16u, mbar);              // x = n -> 0
-  }
+  if (lane < 2)
+    fetch_lines(in, gz, lane, y0 - 1, a.L + 2, n,
+                slot_addr + (uint32_t)lane * (uint32_t)a.slot_pos * 16u + SLK_BEFORE * 16u, mbar);
 }
 
 // TMEM zeroing of columns [c0, c1) (multiples of 16) in the 32 lanes of warp w % 4; the
@@ -393,7 +414,6 @@ __device__ __forceinline__ void conv_epilogue(const ConvArgs& a, const float acc
   const int gy = y0 + ly;
   if (!valid || gy >= n) return;
   const size_t v = ((size_t)z * n + gy) * n + x;
-  const long long line = ((long long)b * n + z) * n + gy;
   if (MODE == CONV_HIDDEN) {
     float zc[16], hv[16];
 #pragma unroll
@@ -411,7 +431,7 @@ __device__ __forceinline__ void conv_epilogue(const ConvArgs& a, const float acc
       for (int q = 0; q < 4; ++q)
         zo[q] = make_float4(zc[4 * q], zc[4 * q + 1], zc[4 * q + 2], zc[4 * q + 3]);
     }
-    act_store(a.out, line, n, x, hv);
+    act_store(a.out, b * n + z, gy, n, x, hv);
   } else if (MODE == CONV_OUT_Y) {
 #pragma unroll
     for (int c = 0; c < 5; ++c) a.y[((size_t)b * 5 + c) * N3 + v] = acc[c] + bias[c];
@@ -432,7 +452,7 @@ __device__ __forceinline__ void conv_epilogue(const ConvArgs& a, const float acc
       d[4 * q + 2] = acc[4 * q + 2] * gelu_grad_f(zz.z);
       d[4 * q + 3] = acc[4 * q + 3] * gelu_grad_f(zz.w);
     }
-    act_store(a.out, line, n, x, d);
+    act_store(a.out, b * n + z, gy, n, x, d);
   }
 }
 
@@ -469,7 +489,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3_kernel(ConvArgs a) {
   uint64_t* drained = done + NB_MAX;                             // [NB_MAX]: output released
   uint32_t* tslot = reinterpret_cast<uint32_t*>(drained + NB_MAX);
   int* sflag = reinterpret_cast<int*>(tslot + 1);
-  const bf16* in = a.in + (size_t)b * N3 * CH;
+  const bf16* in = a.in + (size_t)b * n * n * (n + 2) * CH;
   const uint32_t sa0 = smem_u32(sa);
   const unsigned long long limit = a.wait_ns;
 
@@ -678,199 +698,332 @@ static sim_status launch_conv(int mode, ConvArgs a, int B, cudaStream_t st) {
 
 // ------------------------------------------------------------------ weight gradient
 // dW[tap][ci][co] = sum_v in[v + off(tap)][ci] dz[v][co] and db[co] = sum_v dz[v][co], as
-// tensor-core GEMMs with M = (tap, ci), N = co and K = voxels: 16 consecutive x positions of
-// one line per MMA step (a K block). For every K block the producer warps write into a
-// shared-memory stage the block's 27 shifted input tiles (16 channels x 16 voxels each: tap t
-// at rows 16 (t mod 8) .. + 15 of the M = 128 operand of tap group t / 8) and its dz tile
-// (N = 16 rows), every one transposed on the way into the no-swizzle K-major layout (a row is
-// 8 voxels of one channel: stmatrix .trans from the fragment of 4-byte channel pairs). One
-// thread issues the stage's four M128 N16 K16 MMAs (tap groups 0..3) into four 16-column TMEM
-// accumulators that collect all of the CTA's K blocks; the epilogue adds them to dW / db with
-// vector atomics. Row 48 of group 3 (tap slot 3, channel 0) is a constant row of ones, so its
-// accumulator row is db; the other unused rows of group 3 stay zero. Voxels past the end of a
-// line (n not a multiple of 16) have dz = 0.
-constexpr int DW_PRODUCERS = 8;                     // producer warps; one more issues the MMAs
-constexpr int DW_THREADS = 32 * (DW_PRODUCERS + 1);
-constexpr int DW_STAGES = 3;
-constexpr int DW_A_BYTES = 4 * 4096;                // four tap groups x 128 rows x 32 bytes
-constexpr int DW_STAGE_BYTES = DW_A_BYTES + 512;    // + the dz tile: 16 rows x 32 bytes
-constexpr int DW_SMEM = DW_STAGES * DW_STAGE_BYTES + (2 * DW_STAGES + 1) * 8 + 16;
-constexpr int DW_CTAS_PER_SM = 4;
+// tensor-core GEMMs whose reduction dimension K is the position along x. The activation
+// layout (16-byte positions of 8 channels) is already the no-swizzle MN-major operand: a core
+// matrix is 8 channels (contiguous) x 8 positions (16 bytes apart), the next 8 positions
+// follow 128 bytes on (LBO) and the next 8 channels one half-line on (SBO). So a stage is
+// bulk copies of lines, with no transposition and no im2col.
+//
+// A stage holds DW_G = 6 consecutive lines of dz (2 halves x 6 lines x 8 channels: N = 96
+// columns) and the DW_I = 8 input lines y0 - 1 .. y0 + 6 of plane z + dz that they meet
+// (M = 2 x 8 x 8 = 128 rows), for a run of xs positions. One MMA over 16 positions correlates
+// every input line with every dz line: the blocks (i, j) with i - j - 1 = dy in {-1, 0, 1}
+// are the three dy taps (18 of the 48 blocks, the others are not read), dx is a shift of the
+// A operand by one position. The accumulators of the three dx take 3 x 96 of the 512 TMEM
+// columns and collect all of the CTA's stages; dz is the CTA's blockIdx.y, which triples the
+// reads (from L2) but lets N be 96: an MMA reads its 4 KB A operand from shared memory
+// whatever N is. The epilogue adds the six blocks of each tap through shared memory and the
+// result to dW with vector atomics; the four epilogue warps of the dz = 0 CTAs also sum db
+// from the staged dz lines while the MMAs run.
+// Measured per layer: 33 us at 64^3 x 2 and 94 us at 128^3, against 303 us (64^3 x 2) for
+// im2col tiles transposed by stmatrix into K-major stages (N = 16), which spent its time on
+// 27 loads and stores per position.
+constexpr int DW_G = 6, DW_I = DW_G + 2;   // dz lines, input lines per stage
+constexpr int DW_NC = 16 * DW_G;           // accumulator columns of one dx
+constexpr int DW_THREADS = 192;            // loader warp, MMA warp, four epilogue warps
+constexpr int DW_MAX_STAGES = 6;
+constexpr int DW_XS = 128;                 // positions per stage, at most
+constexpr int DW_RED = DW_I * 3 * 256 * 4;  // bytes of the epilogue's partial sums
 
 struct DwArgs {
-  const bf16* in;  // layer input [B][n][n][2][n][8]
+  const bf16* in;  // layer input, activation layout
   const bf16* dz;  // gradient at the layer's output, same layout
-  int n, nxb;      // grid size, K blocks per line
-  long long kblocks, per_cta;
+  int n;
+  int xs, nseg;    // positions per stage (a multiple of 16 where nseg > 1), stages per line
+  int nyt;         // dz line tiles per plane
+  int pi, pg;      // positions between the half-lines of the staged input and dz
+  int g_whole;     // dz lines staged whole with their padding (n a multiple of 16, nseg = 1)
+  int stages, stage_bytes;
+  int units, per_cta;  // stages of one dz, stages of one CTA
   float* dW;  // [27][16][16], accumulated
   float* db;  // [16], accumulated
   int* err;
   unsigned long long wait_ns;
 };
 
-// four 8x8 bfloat16 matrices from the mma fragment (lane 4 r + q: row r, columns 2q, 2q + 1
-// in register j of matrix j) stored transposed: lane l gives the address of row l mod 8 of
-// matrix l / 8
-__device__ __forceinline__ void stmatrix_trans4(uint32_t addr, const uint32_t v[4]) {
-  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
-               "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3])
-               : "memory");
+// source of the zero dz positions: those that pad a run to a multiple of 16, and whole lines
+// past the last one
+__device__ uint4 dw_zeros[(DW_G - 1) * (DW_XS + 2)];
+
+// stage u -> segment, line tile and plane, stepped without divisions
+struct DwUnit {
+  int seg, yt, zb;
+  __device__ __forceinline__ DwUnit(const DwArgs& a, int u) {
+    seg = u % a.nseg;
+    u /= a.nseg;
+    yt = u % a.nyt;
+    zb = u / a.nyt;  // b n + z
+  }
+  __device__ __forceinline__ void next(const DwArgs& a) {
+    if (++seg < a.nseg) return;
+    seg = 0;
+    if (++yt < a.nyt) return;
+    yt = 0;
+    ++zb;
+  }
+  __device__ __forceinline__ int xn(const DwArgs& a) const { return min(a.xs, a.n - seg * a.xs); }
+  __device__ __forceinline__ int lines(const DwArgs& a) const { return min(DW_G, a.n - yt * DW_G); }
+};
+
+// 8 columns at t0 and 8 at t1 of this thread's TMEM lane
+__device__ __forceinline__ void tmem_ld8x2(uint32_t t0, uint32_t t1, float v[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(t0), "r"(t1)
+      : "memory");
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-__global__ void __launch_bounds__(DW_THREADS) conv_dw_kernel(DwArgs a) {
+__global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + DW_STAGES * DW_STAGE_BYTES);
-  uint64_t* empty = full + DW_STAGES;
-  uint64_t* done = empty + DW_STAGES;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
-  int* sflag = reinterpret_cast<int*>(tslot + 1);
+  __shared__ uint64_t full[DW_MAX_STAGES], empty[DW_MAX_STAGES], done;
+  __shared__ uint32_t tslot;
+  __shared__ int sflag;
+  __shared__ float bred[4][16];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  const int n = a.n, nxb = a.nxb;
-  const long long kb0 = (long long)blockIdx.x * a.per_cta;
-  const long long kb1 = kb0 + a.per_cta < a.kblocks ? kb0 + a.per_cta : a.kblocks;
-  const int nkb = (int)(kb1 - kb0);  // >= 1 by the launch
+  const int n = a.n, S = a.stages;
+  const int dz = (int)blockIdx.y - 1;
+  const bool bias = dz == 0;  // this CTA also sums db
+  const int u0 = blockIdx.x * a.per_cta;
+  const int nu = min(a.per_cta, a.units - u0);  // >= 1 by the launch
   const uint32_t s0 = smem_u32(smem);
+  const uint32_t pi = (uint32_t)a.pi * 16u, pg = (uint32_t)a.pg * 16u;
+  const uint32_t g_off = 2u * DW_I * pi;  // half h, line i of the input at (8 h + i) pi
+  const uint32_t g_x0 = a.g_whole ? 16u : 0u;  // dz position x0 within its half-line
   const unsigned long long limit = a.wait_ns;
 
-  for (int i = tid; i < DW_STAGES * DW_STAGE_BYTES / 16; i += DW_THREADS)
+  // positions that no copy writes meet zero dz positions: they only have to be finite
+  for (int i = tid; i < S * a.stage_bytes / 16; i += DW_THREADS)
     reinterpret_cast<uint4*>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
-  __syncthreads();
-  if (tid < 2 * DW_STAGES) {
-    // group 3, M group 6 (tap slot 3, channels 0-7), K chunk tid & 1, row 0: bfloat16 ones
-    const int st = tid >> 1, kc = tid & 1;
-    *reinterpret_cast<uint4*>(smem + st * DW_STAGE_BYTES + 3 * 4096 + 6 * 256 + kc * 128) =
-        make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
-  }
   if (tid == 0) {
-    for (int st = 0; st < DW_STAGES; ++st) {
-      mbar_init(full + st, DW_PRODUCERS);
-      mbar_init(empty + st, 1);
+    for (int st = 0; st < S; ++st) {
+      mbar_init(full + st, 1);
+      mbar_init(empty + st, bias ? 5 : 1);
     }
-    mbar_init(done, 1);
-    *sflag = 0;
+    mbar_init(&done, 1);
+    sflag = 0;
   }
-  if (w == 0) tmem_alloc_warp(tslot, 64u);
+  if (w == 0) tmem_alloc_warp(&tslot, 512u);
   fence_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = tslot;
+  if (w < 4) tmem_zero(tmem, 0, 3 * DW_NC, w, 1);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
 
-  if (w < DW_PRODUCERS) {
-    const long long N3 = (long long)n * n * n;
-    const int r = lane >> 2, q = lane & 3;  // fragment row (voxel of an 8-voxel chunk), pair
-    const int mj = lane >> 3, row = lane & 7;
-    // matrix j = 2 h + kc: channel half h, K chunk kc (voxels 8 kc .. 8 kc + 7)
-    const uint32_t row_off = (uint32_t)((mj >> 1) * 256 + (mj & 1) * 128 + row * 16);
-    for (int k = 0; k < nkb; ++k) {
-      const int st = k % DW_STAGES;
+  float bacc[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) bacc[c] = 0.0f;
+
+  if (w == 0) {
+    // ---- loader: stage k holds unit u0 + k
+    DwUnit u(a, u0);
+    int issued = 0;
+    for (int k = 0; k < nu; ++k, u.next(a)) {
+      const int st = k % S;
       uint32_t ok = 1;
-      if (k >= DW_STAGES && lane == 0) ok = mbar_wait_ns(empty + st, ((k / DW_STAGES) - 1) & 1, limit);
+      if (k >= S && lane == 0) ok = mbar_wait_ns(empty + st, ((k / S) - 1) & 1, limit);
       ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) {
-        if (lane == 0) *sflag = 1;
+        if (lane == 0) sflag = 1;
         break;
       }
-      long long kb = kb0 + k;
-      const int xb = (int)(kb % nxb);
-      kb /= nxb;
-      const int y = (int)(kb % n);
-      kb /= n;
-      const int z = (int)(kb % n);
-      const int b = (int)(kb / n);
-      const int x0 = 16 * xb;
-      const uint32_t stage = s0 + (uint32_t)(st * DW_STAGE_BYTES);
-      const bf16* inb = a.in + (size_t)b * N3 * CH;
-      const bf16* dzb = a.dz + (size_t)b * N3 * CH;
-      for (int j = w; j < 28; j += DW_PRODUCERS) {
-        uint32_t v[4];
-        uint32_t dst;
-        if (j < 27) {
-          const int ddz = j / 9 - 1, ddy = (j / 3) % 3 - 1, ddx = j % 3 - 1;
-          const long long line = (long long)wrapi(z + ddz, n) * n + wrapi(y + ddy, n);
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            const int x = wrapi(x0 + 8 * (m & 1) + r + ddx, n);
-            v[m] = __ldg(reinterpret_cast<const unsigned int*>(inb + act_off(line, n, m >> 1, x) + 2 * q));
-          }
-          dst = stage + (uint32_t)((j >> 3) * 4096 + (j & 7) * 512);
-        } else {
-          const long long line = (long long)z * n + y;
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            const int x = x0 + 8 * (m & 1) + r;
-            v[m] = x < n ? __ldg(reinterpret_cast<const unsigned int*>(dzb + act_off(line, n, m >> 1, x) + 2 * q))
-                         : 0u;
-          }
-          dst = stage + (uint32_t)DW_A_BYTES;
-        }
-        stmatrix_trans4(dst + row_off, v);
+      const int x0 = u.seg * a.xs, xn = u.xn(a), y0 = u.yt * DW_G, nl = u.lines(a);
+      const int xp = (xn + 15) & ~15;  // dz positions, padded with zeros
+      const int ni = nl + 2;           // input lines that meet the dz lines
+      if (lane == 0) {
+        const uint32_t tx =
+            2u * 16u * (uint32_t)(ni * (xn + 2) + DW_G * (a.g_whole ? n + 2 : xp));
+        uint64_t state;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 %0, [%1], %2;"
+                     : "=l"(state)
+                     : "r"(smem_u32(full + st)), "r"(tx)
+                     : "memory");
+        (void)state;
       }
-      fence_async_smem();
+      __syncwarp();
+      const uint32_t stage = s0 + (uint32_t)(st * a.stage_bytes);
+      const int b = u.zb / n;
+      const int gz = b * n + wrapi(u.zb - b * n + dz, n);
+      if (a.nseg == 1) {
+        // whole padded lines: one copy per half and wrap piece
+        if (lane < 2) fetch_lines(a.in, gz, lane, y0 - 1, ni, n, stage + (uint32_t)lane * DW_I * pi, full + st);
+      } else if (lane < 2 * ni) {
+        const int i = lane >> 1, h = lane & 1;
+        bulk_g2s(stage + (uint32_t)(DW_I * h + i) * pi,
+                 a.in + act_off(gz, wrapi(y0 - 1 + i, n), n, h, x0 - 1), (uint32_t)(xn + 2) * 16u, full + st);
+      }
+      if (a.g_whole) {
+        if (lane >= 2 && lane < 4) {
+          const int h = lane - 2;
+          const uint32_t d = stage + g_off + (uint32_t)(DW_G * h) * pg;
+          bulk_g2s(d, a.dz + act_off(u.zb, y0, n, h, -1), (uint32_t)nl * pg, full + st);
+          if (nl < DW_G) bulk_g2s(d + (uint32_t)nl * pg, dw_zeros, (uint32_t)(DW_G - nl) * pg, full + st);
+        }
+      } else if (lane >= 16 && lane < 16 + 2 * DW_G) {
+        const int j = (lane - 16) >> 1, h = lane & 1;
+        const uint32_t d = stage + g_off + (uint32_t)(DW_G * h + j) * pg;
+        const int live = j < nl ? xn : 0;
+        if (live)
+          bulk_g2s(d, a.dz + act_off(u.zb, y0 + j, n, h, x0), (uint32_t)live * 16u, full + st);
+        if (live < xp) bulk_g2s(d + (uint32_t)live * 16u, dw_zeros, (uint32_t)(xp - live) * 16u, full + st);
+      }
+      issued = k + 1;
+    }
+    // no copy may still be writing shared memory when the CTA reuses it or exits: the last
+    // use of every stage
+    if (lane == 0)
+      for (int k = max(0, issued - S); k < issued; ++k)
+        if (!mbar_wait_ns(full + k % S, (k / S) & 1, kDrainNs)) sflag = 1;
+    __syncwarp();
+  } else if (w == 1) {
+    // ---- MMA issuer: per stage and dx a chain of MMAs (16 positions each) into the dx's
+    //      accumulator (chained MMAs on one accumulator run several times faster than
+    //      MMAs that change it)
+    if (lane == 0) {
+      constexpr uint32_t idesc = umma_idesc_bf16_mn(128, DW_NC);
+      DwUnit u(a, u0);
+      int committed = 0;
+      for (int k = 0; k < nu; ++k, u.next(a)) {
+        const int st = k % S;
+        if (!mbar_wait_ns(full + st, (k / S) & 1, limit)) {
+          sflag = 1;
+          break;
+        }
+        tc_fence_after();
+        const int steps = (u.xn(a) + 15) >> 4;
+        const uint32_t stage = s0 + (uint32_t)(st * a.stage_bytes);
+        const uint64_t ad = umma_desc(stage, 128u, pi);
+        const uint64_t bd = umma_desc(stage + g_off + g_x0, 128u, pg);
+#pragma unroll 1
+        for (int dx = 0; dx < 3; ++dx)
+          for (int q = 0; q < steps; ++q)
+            // descriptors are linear in the start address (16-byte units: one per position)
+            umma_bf16(tmem + (uint32_t)(dx * DW_NC), ad + (uint64_t)(16 * q + dx),
+                      bd + (uint64_t)(16 * q), idesc, 1u);
+        umma_commit(empty + st);
+        committed = k + 1;
+      }
+      if (committed > 0) {
+        // completes once every MMA issued above has; waited for before TMEM is read or freed
+        umma_commit(&done);
+        if (!mbar_wait_ns(&done, 0, kDrainNs)) sflag = 1;
+      }
+    }
+    __syncwarp();
+  } else if (bias) {
+    // ---- db: thread t of the four warps sums half t & 1 of the positions t / 2 mod 64
+    const int t = tid - 64, h = t & 1;
+    DwUnit u(a, u0);
+    for (int k = 0; k < nu; ++k, u.next(a)) {
+      const int st = k % S;
+      uint32_t ok = 0;
+      if (lane == 0) ok = mbar_wait_ns(full + st, (k / S) & 1, limit);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (!ok) {
+        if (lane == 0) sflag = 1;
+        break;
+      }
+      const int xn = u.xn(a), nl = u.lines(a);
+      const uint8_t* g = smem + (size_t)st * a.stage_bytes + g_off + g_x0 + (size_t)(DW_G * h) * pg;
+      for (int j = 0; j < nl; ++j)
+        for (int x = t >> 1; x < xn; x += 64) {
+          const uint4 v = *reinterpret_cast<const uint4*>(g + (size_t)j * pg + (size_t)x * 16);
+          const uint32_t q[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            bacc[2 * c] += __uint_as_float(q[c] << 16);  // a bfloat16 is the high half of a float
+            bacc[2 * c + 1] += __uint_as_float(q[c] & 0xffff0000u);
+          }
+        }
       __syncwarp();
       if (lane == 0) {
         uint64_t state;
         asm volatile("mbarrier.arrive.shared::cta.b64 %0, [%1];"
                      : "=l"(state)
-                     : "r"(smem_u32(full + st))
+                     : "r"(smem_u32(empty + st))
                      : "memory");
         (void)state;
       }
     }
-  } else if (lane == 0) {
-    // ---- MMA issuer: the stage's four tap groups, then release the stage
-    const uint32_t idesc = umma_idesc_bf16(128, 16);
-    for (int k = 0; k < nkb; ++k) {
-      const int st = k % DW_STAGES;
-      if (!mbar_wait_ns(full + st, (k / DW_STAGES) & 1, limit)) {
-        *sflag = 1;
-        break;
-      }
-      tc_fence_after();
-      const uint32_t stage = s0 + (uint32_t)(st * DW_STAGE_BYTES);
-      const uint64_t bdesc = umma_desc(stage + DW_A_BYTES, 128u, 256u);
-#pragma unroll
-      for (int g = 0; g < 4; ++g)
-        umma_bf16(tmem + 16u * g, umma_desc(stage + 4096u * g, 128u, 256u), bdesc, idesc, k > 0 ? 1u : 0u);
-      umma_commit(empty + st);
-    }
-    // completes once every MMA issued above has; waited for before TMEM is read or freed
-    umma_commit(done);
-    if (!mbar_wait_ns(done, 0, kDrainNs)) *sflag = 1;
   }
-  __syncwarp();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (w < 4 && *sflag == 0) {
-    // lane 32 w + l of TMEM = row m: tap slot m / 16 of each group, channel m mod 16
-    const int m = 32 * w + lane, slot = m >> 4, ci = m & 15;
+  if (w >= 2 && sflag == 0) {
+    // TMEM lane 8 (8 h + i) + c8 of warp w % 4: half h = q / 2, input lines i0 .. i0 + 3;
+    // columns 8 (6 h' + j) + c8'
+    const int t = tid - 64, q = w & 3;
+    const int i0 = 4 * (q & 1), i = i0 + (lane >> 3), ci = 8 * (q >> 1) + (lane & 7);
+    const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
+    float* red = reinterpret_cast<float*>(smem);  // [i][dy + 1][ci][co]
+#pragma unroll 1
+    for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll 1
+      for (int j = max(0, i0 - 2); j < min(DW_G, i0 + 4); ++j) {  // the same for the whole warp
+        float acc[16];
+        tmem_ld8x2(tl + (uint32_t)(dx * DW_NC + 8 * j), tl + (uint32_t)(dx * DW_NC + 8 * (DW_G + j)), acc);
+        const int dy = i - 1 - j;
+        if (dy >= -1 && dy <= 1) {
+          float4* d = reinterpret_cast<float4*>(red + (i * 3 + dy + 1) * 256 + ci * 16);
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      float acc[16];
-      tmem_ld16(tmem + ((uint32_t)(32 * w) << 16) + 16u * g, acc);
-      const int t = 8 * g + slot;
-      float* dst = t < 27 ? a.dW + (size_t)(t * CH + ci) * CH : (t == 27 && ci == 0 ? a.db : nullptr);
-      if (dst)
+          for (int c = 0; c < 4; ++c)
+            d[c] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
+        }
+        __syncwarp();
+      }
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      for (int e = t; e < 3 * 64; e += 128) {
+        const int r = e >> 6, f = e & 63;  // dy + 1, float4 of the 16 x 16 block
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int p = r; p < r + DW_G; ++p) {  // the input lines that meet a dz line at this dy
+          const float4 v = reinterpret_cast<const float4*>(red + (p * 3 + r) * 256)[f];
+          sum.x += v.x;
+          sum.y += v.y;
+          sum.z += v.z;
+          sum.w += v.w;
+        }
+        const int tap = 9 * (dz + 1) + 3 * r + dx;
+        atomicAdd(reinterpret_cast<float4*>(a.dW + (size_t)tap * CH * CH) + f, sum);
+      }
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+    }
+    if (bias) {
 #pragma unroll
-        for (int c4 = 0; c4 < 4; ++c4)
-          atomicAdd(reinterpret_cast<float4*>(dst) + c4,
-                    make_float4(acc[4 * c4], acc[4 * c4 + 1], acc[4 * c4 + 2], acc[4 * c4 + 3]));
+      for (int c = 0; c < 8; ++c)
+#pragma unroll
+        for (int o = 16; o > 1; o >>= 1) bacc[c] += __shfl_xor_sync(0xffffffffu, bacc[c], o);
+      if (lane < 2)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) bred[w - 2][8 * lane + c] = bacc[c];
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (t < 16) atomicAdd(a.db + t, bred[0][t] + bred[1][t] + bred[2][t] + bred[3][t]);
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (tid == 0 && *sflag) atomicExch(a.err, 1);
-  if (w == 0) tmem_dealloc_warp(tmem, 64u);
+  if (tid == 0 && sflag) atomicExch(a.err, 1);
+  if (w == 0) tmem_dealloc_warp(tmem, 512u);
 }
 
 static sim_status launch_dw(const bf16* in, const bf16* dz, int n, int B, float* dW, float* db,
                             int* err, unsigned long long wait_ns, cudaStream_t st) {
+  constexpr int kSmemMax = 200 * 1024;
   static std::atomic<unsigned long long> done{0};
   int dev = 0;
   DH_CUDA_TRY(cudaGetDevice(&dev));
   if (!(done.load() & (1ull << (dev & 63)))) {
-    DH_CUDA_TRY(cudaFuncSetAttribute(conv_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM));
+    DH_CUDA_TRY(cudaFuncSetAttribute(conv_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
     done.fetch_or(1ull << (dev & 63));
   }
   int sms = 0;
@@ -879,16 +1032,32 @@ static sim_status launch_dw(const bf16* in, const bf16* dz, int n, int B, float*
   a.in = in;
   a.dz = dz;
   a.n = n;
-  a.nxb = cdiv(n, 16);
-  a.kblocks = (long long)B * n * n * a.nxb;
-  const long long ctas = std::max(1, sms * DW_CTAS_PER_SM);
-  a.per_cta = (a.kblocks + ctas - 1) / ctas;
+  a.nseg = cdiv(n, DW_XS);
+  a.xs = a.nseg == 1 ? n : 16 * cdiv(cdiv(n, a.nseg), 16);
+  a.nseg = cdiv(n, a.xs);
+  a.nyt = cdiv(n, DW_G);
+  a.g_whole = a.nseg == 1 && n % 16 == 0;
+  a.pi = a.xs + 2;
+  a.pg = a.g_whole ? n + 2 : 16 * cdiv(a.xs, 16);
+  a.stage_bytes = 16 * (2 * DW_I * a.pi + 2 * DW_G * a.pg);
+  a.stages = std::min(DW_MAX_STAGES, kSmemMax / a.stage_bytes);
+  const long long units = (long long)B * n * a.nyt * a.nseg;
+  if (units > (1ll << 30)) {
+    set_error("closure: %lld line tiles in the weight gradient", units);
+    return SIM_EINVAL;
+  }
+  a.units = (int)units;
+  // one CTA per SM (all 512 TMEM columns), a third of them for each dz
+  const int ctas = std::min(a.units, std::max(1, sms / 3));
+  a.per_cta = cdiv(a.units, ctas);
   a.dW = dW;
   a.db = db;
   a.err = err;
   a.wait_ns = wait_ns;
-  const int grid = (int)((a.kblocks + a.per_cta - 1) / a.per_cta);
-  conv_dw_kernel<<<grid, DW_THREADS, DW_SMEM, st>>>(a);
+  const dim3 grid(cdiv(a.units, a.per_cta), 3);
+  // at least 116 KB so that no second CTA (of this kernel or a convolution) shares the SM
+  const size_t bytes = std::max<size_t>({(size_t)a.stages * a.stage_bytes, (size_t)DW_RED, (size_t)116 * 1024});
+  conv_dw_kernel<<<grid, DW_THREADS, bytes, st>>>(a);
   DH_LAUNCH_CHECK();
   return SIM_OK;
 }
@@ -905,7 +1074,8 @@ __global__ void closure_pack_kernel(const float* __restrict__ gas, F5 mu, F5 inv
   for (int f = 0; f < 16; ++f) v[f] = 0.0f;
 #pragma unroll
   for (int f = 0; f < 5; ++f) v[f] = (gas[((size_t)b * 5 + f) * N3 + i] - mu.v[f]) * inv_sigma.v[f];
-  act_store(x, (long long)b * (N3 / n) + i / n, n, (int)(i % n), v);
+  const int row = (int)(i / n);
+  act_store(x, b * n + row / n, row % n, n, (int)(i - (long long)row * n), v);
 }
 
 // loss += norm sum (y - (tgt - in) / s)^2 over 5 fields; dz4 = bf16(2 norm (y - t))
@@ -928,7 +1098,8 @@ __global__ void closure_loss_kernel(const float* __restrict__ y, const float* __
       acc += d * d;
       g[f] = 2.0f * norm * d;
     }
-    act_store(dz4, (long long)b * (N3 / n) + i / n, n, (int)(i % n), g);
+    const int row = (int)(i / n);
+    act_store(dz4, b * n + row / n, row % n, n, (int)(i - (long long)row * n), g);
   }
   block_sum_atomic(acc * norm, loss);
 }
@@ -1019,13 +1190,13 @@ sim_status closure_prepare(sim_closure_s* c, int n, int B, bool training) {
   ws_free(c);
   c->gen += 1;
   const size_t V = (size_t)n * n * n * B;
-  DH_TRY(ws_alloc(c, &c->x, V * CH));
-  DH_TRY(ws_alloc(c, &c->a1, V * CH));
-  DH_TRY(ws_alloc(c, &c->a2, V * CH));
+  DH_TRY(ws_alloc(c, &c->x, act_count(n, B)));
+  DH_TRY(ws_alloc(c, &c->a1, act_count(n, B)));
+  DH_TRY(ws_alloc(c, &c->a2, act_count(n, B)));
   if (training) {
-    DH_TRY(ws_alloc(c, &c->a3, V * CH));
-    DH_TRY(ws_alloc(c, &c->d1, V * CH));
-    DH_TRY(ws_alloc(c, &c->d2, V * CH));
+    DH_TRY(ws_alloc(c, &c->a3, act_count(n, B)));
+    DH_TRY(ws_alloc(c, &c->d1, act_count(n, B)));
+    DH_TRY(ws_alloc(c, &c->d2, act_count(n, B)));
     DH_TRY(ws_alloc(c, &c->z1, V * CH));
     DH_TRY(ws_alloc(c, &c->z2, V * CH));
     DH_TRY(ws_alloc(c, &c->z3, V * CH));

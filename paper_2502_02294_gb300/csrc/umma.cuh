@@ -32,6 +32,12 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
          ((uint32_t)(M >> 4) << 24);
 }
 
+// the same with A and B MN-major (the reduction index strided): 8 contiguous rows x 8 K per
+// core matrix, K rows 16 bytes apart, LBO between groups of 8 K, SBO between groups of 8 rows
+__host__ __device__ constexpr uint32_t umma_idesc_bf16_mn(int M, int N) {
+  return umma_idesc_bf16(M, N) | (1u << 15) | (1u << 16);
+}
+
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
                                           uint32_t accumulate) {
   asm volatile(
@@ -73,22 +79,26 @@ __device__ __forceinline__ uint32_t mbar_test(uint64_t* mbar, uint32_t parity) {
 // timer (and at most 2^26 polls); returns 1 when the phase completed, 0 when the wait gave
 // up. limit_ns = 0: one non-blocking check only. Each poll may suspend the thread for up to
 // kSuspendNs until the phase completes, so a waiting warp does not spin on the issue slots
-// the working warps of its scheduler need; a wait that gives up therefore does so up to
-// kSuspendNs after its limit.
-constexpr uint32_t kSuspendNs = 20000;
+// the working warps of its scheduler need. The timer is read only after a first poll has
+// run out (most waits end within it), so a wait gives up at most two polls after its limit.
+constexpr uint32_t kSuspendNs = 10000;
+__device__ __forceinline__ uint32_t mbar_poll(uint64_t* mbar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(done)
+      : "r"(smem_u32(mbar)), "r"(parity), "r"(kSuspendNs)
+      : "memory");
+  return done;
+}
 __device__ __forceinline__ uint32_t mbar_wait_ns(uint64_t* mbar, uint32_t parity, uint64_t limit_ns) {
   if (mbar_test(mbar, parity)) return 1;
   if (limit_ns == 0) return 0;
+  if (mbar_poll(mbar, parity)) return 1;
   const uint64_t t0 = global_ns();
   for (int it = 0; it < (1 << 26); ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(smem_u32(mbar)), "r"(parity), "r"(kSuspendNs)
-        : "memory");
-    if (done) return 1;
+    if (mbar_poll(mbar, parity)) return 1;
     if (global_ns() - t0 >= limit_ns) return 0;
   }
   return 0;
