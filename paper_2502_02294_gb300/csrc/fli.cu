@@ -163,39 +163,8 @@ __global__ void axpby_kernel(float alpha, const float* __restrict__ x, float bet
 }
 
 // ------------------------------------------------------------------ r_c(k)
-// One pass over the half spectra of X and Y: per bin the mode weight, weight * |k| and the
-// three weighted powers |X|^2, |Y|^2, Re(X conj Y) (FP64 histograms in shared memory).
-__global__ void xc_bin_kernel(const cufftComplex* __restrict__ a, const cufftComplex* __restrict__ b,
-                              int n, int nbins, double* __restrict__ sums) {
-  pdl_enter();
-  extern __shared__ double hist[];  // 5 * nbins
-  for (int j = threadIdx.x; j < 5 * nbins; j += blockDim.x) hist[j] = 0.0;
-  __syncthreads();
-  const int nh = n / 2 + 1;
-  const long long NC = (long long)n * n * nh;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < NC;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int kx = (int)(i % nh);
-    const long long r = i / nh;
-    int ky = (int)(r % n), kz = (int)(r / n);
-    if (ky > n / 2) ky -= n;
-    if (kz > n / 2) kz -= n;
-    const double kk = sqrt((double)kx * kx + (double)ky * ky + (double)kz * kz);
-    const int bin = (int)rint(kk);
-    if (bin < 1 || bin > nbins) continue;
-    const double w = (kx == 0 || (n % 2 == 0 && kx == n / 2)) ? 1.0 : 2.0;
-    const cufftComplex x = a[i], y = b[i];
-    atomicAdd(&hist[bin - 1], w);
-    atomicAdd(&hist[nbins + bin - 1], w * kk);
-    atomicAdd(&hist[2 * nbins + bin - 1], w * ((double)x.x * x.x + (double)x.y * x.y));
-    atomicAdd(&hist[3 * nbins + bin - 1], w * ((double)y.x * y.x + (double)y.y * y.y));
-    atomicAdd(&hist[4 * nbins + bin - 1], w * ((double)x.x * y.x + (double)x.y * y.y));
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < 5 * nbins; j += blockDim.x)
-    if (hist[j] != 0.0) atomicAdd(&sums[j], hist[j]);
-}
-
+// (spectrum_bin_kernel sums per bin the mode weight, weight * |k| and the three weighted powers
+// |X|^2, |Y|^2, Re(X conj Y))
 __global__ void xc_finish_kernel(const double* __restrict__ sums, int nbins, double kf,
                                  double* __restrict__ k, double* __restrict__ rc,
                                  double* __restrict__ nm) {
@@ -276,16 +245,7 @@ extern "C" sim_status sim_cross_correlation(const float* a, const float* b, int3
     set_error("cufftExecR2C failed");
     r = SIM_ECUDA;
   }
-  if (r == SIM_OK) {
-    int blocks = cdiv(NC, 256);
-    if (blocks > 152 * 4) blocks = 152 * 4;
-    DH_CUDA_TRY((launch_pdl(xc_bin_kernel, blocks, 256, 5 * nbins * sizeof(double), st, buf, buf + NC, n, nbins, sums)));
-    count_launch();
-    if (cudaGetLastError() != cudaSuccess) {
-      set_error("xc_bin_kernel launch failed");
-      r = SIM_ECUDA;
-    }
-  }
+  if (r == SIM_OK) r = launch_spectrum_bins(buf, buf + NC, n, nbins, 3, sums, st);
   if (r == SIM_OK) {
     DH_CUDA_TRY((launch_pdl(xc_finish_kernel, cdiv(nbins, 128), 128, 0, st, sums, nbins, 2.0 * M_PI / box, k, rc, nmodes)));
     count_launch();

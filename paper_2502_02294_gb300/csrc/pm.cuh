@@ -24,6 +24,12 @@ struct FFTPlans {
 // Plans (batch 1) shared by the standalone entry points, keyed by n (created on first use).
 FFTPlans* shared_plans(int n);
 
+// Per bin 1 .. nbins of |k| (half spectra of n^3 fields): mode weight, weight |k|, and
+// `powers` weighted powers (1: Re(a conj b); 3: |a|^2, |b|^2, Re(a conj b)) accumulated into
+// sums [2 + powers][nbins]; powers = 0: the weights alone, [nbins] (a, b unused).
+sim_status launch_spectrum_bins(const cufftComplex* a, const cufftComplex* b, int n, int nbins,
+                                int powers, double* sums, cudaStream_t st);
+
 // ------------------------------------------------------------------ launchers
 // Every launcher below runs B instances of one grid size at once; array arguments hold the
 // instances one after another (see SArg / DPart in common.cuh).
