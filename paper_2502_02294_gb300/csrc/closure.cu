@@ -139,43 +139,45 @@ static ConvGeom conv_geom(int n, int B) {
 // erfc(|x|) ~ (a1 t + a2 t^2 + a3 t^3 + a4 t^4 + a5 t^5) e^{-x^2}. Branch-free; e receives
 // e^{-x^2}. 1 + erf(x) is then 2 - erfc(|x|) for x >= 0 and erfc(|x|) for x < 0, without
 // cancellation on the negative side.
-__device__ __forceinline__ float erfc_abs(float ax, float& e) {
-  const float t = __fdividef(1.0f, fmaf(0.3275911f, ax, 1.0f));
-  e = __expf(-ax * ax);
-  const float poly =
-      fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f),
-           0.254829592f);
-  return t * poly * e;
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
-
-// GELU(z) = z Phi(z) = z (1 + erf(z / sqrt 2)) / 2, on two values with packed float32
-// arithmetic (FFMA2 / FMUL2)
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ float2 ff2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 gelu2_f(float2 z) {
+// q = erfc(|z| / sqrt 2) and e = e^{-z^2 / 2} of two values, packed float32 arithmetic (FFMA2 /
+// FMUL2); the denormal-flushing approximations are one instruction each
+__device__ __forceinline__ float2 erfc2(float2 z, float2& e) {
   const float2 x = __fmul2_rn(z, ff2(0.70710678118654752f));
-  const float2 ax = make_float2(fabsf(x.x), fabsf(x.y));
-  const float2 den = __ffma2_rn(ff2(0.3275911f), ax, ff2(1.0f));
-  const float2 t = make_float2(__fdividef(1.0f, den.x), __fdividef(1.0f, den.y));
-  const float2 x2 = __fmul2_rn(ax, ax);
-  const float2 e = make_float2(__expf(-x2.x), __expf(-x2.y));
+  const float2 den = __ffma2_rn(ff2(0.3275911f), make_float2(fabsf(x.x), fabsf(x.y)), ff2(1.0f));
+  const float2 t = make_float2(rcp_ftz(den.x), rcp_ftz(den.y));
+  const float2 y = __fmul2_rn(__fmul2_rn(x, x), ff2(-1.4426950408889634f));
+  e = make_float2(ex2_ftz(y.x), ex2_ftz(y.y));
   float2 poly = __ffma2_rn(t, ff2(1.061405429f), ff2(-1.453152027f));
   poly = __ffma2_rn(t, poly, ff2(1.421413741f));
   poly = __ffma2_rn(t, poly, ff2(-0.284496736f));
   poly = __ffma2_rn(t, poly, ff2(0.254829592f));
-  const float2 q = __fmul2_rn(__fmul2_rn(t, poly), e);
-  // 1 + erf(x) = 2 - q (x >= 0) or q (x < 0)
-  const float2 sg = make_float2(x.x >= 0.0f ? -1.0f : 1.0f, x.y >= 0.0f ? -1.0f : 1.0f);
-  const float2 base = make_float2(x.x >= 0.0f ? 2.0f : 0.0f, x.y >= 0.0f ? 2.0f : 0.0f);
-  const float2 r = __ffma2_rn(sg, q, base);
-  return __fmul2_rn(__fmul2_rn(z, ff2(0.5f)), r);
+  return __fmul2_rn(__fmul2_rn(t, poly), e);
+}
+
+// GELU(z) = z Phi(z) with Phi(z) = 1 - q / 2 (z >= 0) or q / 2 (z < 0): max(z, 0) - |z| q / 2
+__device__ __forceinline__ float2 gelu2_f(float2 z) {
+  float2 e;
+  const float2 h = __fmul2_rn(__fmul2_rn(z, ff2(0.5f)), erfc2(z, e));
+  return make_float2(fmaxf(z.x, 0.0f) - fabsf(h.x), fmaxf(z.y, 0.0f) - fabsf(h.y));
 }
 
 // d GELU / dz = Phi(z) + z phi(z), phi(z) = e^{-z^2 / 2} / sqrt(2 pi)
-__device__ __forceinline__ float gelu_grad_f(float z) {
-  const float x = z * 0.70710678118654752f;
-  float e;
-  const float q = erfc_abs(fabsf(x), e);
-  return 0.5f * (x >= 0.0f ? 2.0f - q : q) + z * 0.3989422804014327f * e;
+__device__ __forceinline__ float2 gelu_grad2_f(float2 z) {
+  float2 e;
+  const float2 q = __fmul2_rn(erfc2(z, e), ff2(0.5f));
+  const float2 phi = make_float2(z.x >= 0.0f ? 1.0f - q.x : q.x, z.y >= 0.0f ? 1.0f - q.y : q.y);
+  return __ffma2_rn(__fmul2_rn(z, ff2(0.3989422804014327f)), e, phi);
 }
 
 __device__ __forceinline__ int wrapi(int i, int n) {
@@ -337,58 +339,51 @@ __device__ __forceinline__ uint32_t acc_col(const ConvArgs& a, int t, int s) {
   return 16u * (uint32_t)(t * a.R + s);
 }
 
-// One run of input plane i (ring slot i mod ring) for every tile: block (dy, dx) of the
-// weights against the input shifted by (dy, dx), into the len consecutive accumulator slots
-// s .. s + len - 1, which hold output planes lo .. lo + len - 1 (relative to z0); output
-// plane i - 2 + k takes rows 16 k .. 16 k + 15 of the B operand (dz = 1 - k).
-__device__ __forceinline__ void conv_issue_run(const ConvArgs& a, int i, int lo, int len, int s,
-                                               uint32_t tmem, uint64_t a_base, uint64_t b_base,
-                                               uint32_t slot_units) {
+// One run of input plane i (ring slot `slot`) for every tile: block (dy, dx) of the weights
+// against the input shifted by (dy, dx), into the len consecutive accumulator slots
+// s .. s + len - 1; output plane i - 2 + k takes rows 16 k .. 16 k + 15 of the B operand
+// (dz = 1 - k), the run starting at k = first. Called by a whole warp.
+__device__ __forceinline__ void conv_issue_run(const ConvArgs& a, uint32_t leader, int slot, int first,
+                                               int len, int s, uint32_t tmem, uint64_t a_base,
+                                               uint64_t b_base, uint32_t slot_units) {
   const int P = a.P, T = a.T;
-  const uint64_t a_slot = a_base + (uint64_t)((i % a.ring) * slot_units);
   const uint32_t idesc = len == 3 ? umma_idesc_bf16(128, 48)
                                   : (len == 2 ? umma_idesc_bf16(128, 32) : umma_idesc_bf16(128, 16));
-  // rows 16 k0 .. of each 1536-byte block: 8-row groups 128 bytes apart (16-byte units)
-  const uint64_t b_run = b_base + (uint64_t)(16 * (lo - (i - 2)));
+  // descriptors are linear in the start address (16-byte units, within the low word); the
+  // shift (dy, dx) = (-1, -1) of the tile's first position, and rows 16 first .. of each
+  // 1536-byte weight block (8-row groups 128 bytes apart)
+  const uint32_t a_hi = (uint32_t)(a_base >> 32), b_hi = (uint32_t)(b_base >> 32);
+  const uint32_t a_lo = (uint32_t)a_base + (uint32_t)slot * slot_units + SLK_BEFORE - 1;
+  const uint32_t b_lo = (uint32_t)b_base + (uint32_t)(16 * first);
   // tile-major: the 9 MMAs of one tile chain into the same accumulator (switching the
   // accumulator between consecutive MMAs costs several times a chained MMA)
+  int ly = 0, c = 0;
   for (int t = 0; t < T; ++t) {
-    int vb;
-    if (a.contig) {
-      vb = 128 * t;
-    } else {
-      const int ly = t / a.tpl;
-      vb = ly * P + 1 + 128 * (t - ly * a.tpl);
-    }
+    const uint32_t at = a_lo + (uint32_t)(a.contig ? 128 * t : ly * P + 1 + 128 * c);
     const uint32_t d = tmem + acc_col(a, t, s);
 #pragma unroll
-    for (int dy = -1; dy <= 1; ++dy) {
+    for (int dy = 0; dy < 3; ++dy)
 #pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int j = (dy + 1) * 3 + (dx + 1);
-        const uint64_t db = b_run + (uint64_t)(j * 96);  // 1536-byte blocks
-        // descriptors are linear in the start address (16-byte units, low 14 bits)
-        const uint64_t da = a_slot + (uint64_t)(SLK_BEFORE + (1 + dy) * P + dx + vb);
-        umma_bf16(d, da, db, idesc, 1u);
-      }
+      for (int dx = 0; dx < 3; ++dx)
+        umma_bf16_acc(leader, d, at + (uint32_t)(dy * P + dx), a_hi, b_lo + 96u * (uint32_t)(3 * dy + dx),
+                      b_hi, idesc);
+    if (++c == a.tpl) {
+      c = 0;
+      ++ly;
     }
   }
 }
 
-// The MMAs of input plane i: output planes max(0, i - 2) .. min(i, nz - 1), in one run, or
-// two where their slots wrap around the end of the ring.
-__device__ __forceinline__ void conv_issue_input(const ConvArgs& a, int i, int nz, uint32_t tmem,
-                                                 uint64_t a_base, uint64_t b_base,
-                                                 uint32_t slot_units) {
+// The MMAs of input plane i (ring slot `slot`): output planes max(0, i - 2) .. min(i, nz - 1),
+// in one run, or two where their slots wrap around the end of the ring.
+__device__ __forceinline__ void conv_issue_input(const ConvArgs& a, uint32_t leader, int i, int slot,
+                                                 int nz, uint32_t tmem, uint64_t a_base,
+                                                 uint64_t b_base, uint32_t slot_units) {
   const int lo = max(0, i - 2), hi = min(i, nz - 1);
-  const int len = hi - lo + 1, s0 = lo % a.R;
-  if (s0 + len <= a.R) {
-    conv_issue_run(a, i, lo, len, s0, tmem, a_base, b_base, slot_units);
-  } else {
-    const int first = a.R - s0;
-    conv_issue_run(a, i, lo, first, s0, tmem, a_base, b_base, slot_units);
-    conv_issue_run(a, i, lo + first, len - first, 0, tmem, a_base, b_base, slot_units);
-  }
+  const int len = hi - lo + 1, s0 = lo % a.R, first = lo - (i - 2);
+  const int n0 = min(len, a.R - s0);
+  conv_issue_run(a, leader, slot, first, n0, s0, tmem, a_base, b_base, slot_units);
+  if (n0 < len) conv_issue_run(a, leader, slot, first + n0, len - n0, 0, tmem, a_base, b_base, slot_units);
 }
 
 // Epilogue of row r of tile t of output plane z (all 16 channels).
@@ -447,10 +442,14 @@ __device__ __forceinline__ void conv_epilogue(const ConvArgs& a, const float acc
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float4 zz = __ldg(zp + q);
-      d[4 * q] = acc[4 * q] * gelu_grad_f(zz.x);
-      d[4 * q + 1] = acc[4 * q + 1] * gelu_grad_f(zz.y);
-      d[4 * q + 2] = acc[4 * q + 2] * gelu_grad_f(zz.z);
-      d[4 * q + 3] = acc[4 * q + 3] * gelu_grad_f(zz.w);
+      const float2 g0 = gelu_grad2_f(make_float2(zz.x, zz.y));
+      const float2 g1 = gelu_grad2_f(make_float2(zz.z, zz.w));
+      const float2 d0 = __fmul2_rn(make_float2(acc[4 * q], acc[4 * q + 1]), g0);
+      const float2 d1 = __fmul2_rn(make_float2(acc[4 * q + 2], acc[4 * q + 3]), g1);
+      d[4 * q] = d0.x;
+      d[4 * q + 1] = d0.y;
+      d[4 * q + 2] = d1.x;
+      d[4 * q + 3] = d1.y;
     }
     act_store(a.out, b * n + z, gy, n, x, d);
   }
@@ -555,30 +554,29 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3_kernel(ConvArgs a) {
       __syncwarp();
     }
   } else if (w == 2) {
-    // ---- MMA issuer
-    if (lane == 0) {
-      const uint64_t a_base = umma_desc(sa0, (uint32_t)a.slot_pos * 16u, 128u);
-      const uint64_t b_base = umma_desc(smem_u32(sw), 768u, 128u);
-      const uint32_t slot_units = slot_bytes >> 4;
-      int committed = 0;
-      for (int i = 0; i < nin; ++i) {
-        // the slot of output plane i last held output plane i - R
-        if (i < nz && i >= R && !mbar_wait_ns(drained + (i - R), 0, limit)) {
-          *sflag = 1;
-          break;
-        }
-        if (!mbar_wait_ns(full + i, 0, limit)) {
-          *sflag = 1;
-          break;
-        }
-        tc_fence_after();
-        conv_issue_input(a, i, nz, tmem, a_base, b_base, slot_units);
-        umma_commit(done + i);
-        committed = i + 1;
+    // ---- MMA issuer: the whole warp runs the loop, one elected lane issues
+    const uint32_t leader = elect_one();
+    const uint64_t a_base = umma_desc(sa0, (uint32_t)a.slot_pos * 16u, 128u);
+    const uint64_t b_base = umma_desc(smem_u32(sw), 768u, 128u);
+    const uint32_t slot_units = slot_bytes >> 4;
+    int committed = 0, slot = 0;
+    for (int i = 0; i < nin; ++i) {
+      // the slot of output plane i last held output plane i - R
+      uint32_t ok = 1;
+      if (i < nz && i >= R) ok = mbar_wait_ns(drained + (i - R), 0, limit);
+      if (ok) ok = mbar_wait_ns(full + i, 0, limit);
+      if (!__all_sync(0xffffffffu, ok)) {
+        *sflag = 1;
+        break;
       }
-      // the commit of the last issued input completes once every MMA issued before it has
-      if (committed > 0 && !mbar_wait_ns(done + committed - 1, 0, kDrainNs)) *sflag = 1;
+      tc_fence_after();
+      conv_issue_input(a, leader, i, slot, nz, tmem, a_base, b_base, slot_units);
+      umma_commit(leader, done + i);
+      committed = i + 1;
+      if (++slot == ring) slot = 0;
     }
+    // the commit of the last issued input completes once every MMA issued before it has
+    if (committed > 0 && !mbar_wait_ns(done + committed - 1, 0, kDrainNs)) *sflag = 1;
     __syncwarp();
   } else if (w >= 4) {
     // ---- epilogue: output plane z0 + o is final once input o + 2 is in; its accumulator
@@ -888,37 +886,42 @@ __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
     __syncwarp();
   } else if (w == 1) {
     // ---- MMA issuer: per stage and dx a chain of MMAs (16 positions each) into the dx's
-    //      accumulator (chained MMAs on one accumulator run several times faster than
-    //      MMAs that change it)
-    if (lane == 0) {
-      constexpr uint32_t idesc = umma_idesc_bf16_mn(128, DW_NC);
-      DwUnit u(a, u0);
-      int committed = 0;
-      for (int k = 0; k < nu; ++k, u.next(a)) {
-        const int st = k % S;
-        if (!mbar_wait_ns(full + st, (k / S) & 1, limit)) {
-          sflag = 1;
-          break;
-        }
-        tc_fence_after();
-        const int steps = (u.xn(a) + 15) >> 4;
-        const uint32_t stage = s0 + (uint32_t)(st * a.stage_bytes);
-        const uint64_t ad = umma_desc(stage, 128u, pi);
-        const uint64_t bd = umma_desc(stage + g_off + g_x0, 128u, pg);
-#pragma unroll 1
-        for (int dx = 0; dx < 3; ++dx)
-          for (int q = 0; q < steps; ++q)
-            // descriptors are linear in the start address (16-byte units: one per position)
-            umma_bf16(tmem + (uint32_t)(dx * DW_NC), ad + (uint64_t)(16 * q + dx),
-                      bd + (uint64_t)(16 * q), idesc, 1u);
-        umma_commit(empty + st);
-        committed = k + 1;
+    //      accumulator; the whole warp runs the loop, one elected lane issues
+    constexpr uint32_t idesc = umma_idesc_bf16_mn(128, DW_NC);
+    const uint32_t leader = elect_one();
+    const uint64_t a_base = umma_desc(s0, 128u, pi), b_base = umma_desc(s0 + g_off + g_x0, 128u, pg);
+    const uint32_t a_hi = (uint32_t)(a_base >> 32), b_hi = (uint32_t)(b_base >> 32);
+    int committed = 0, st = 0, par = 0, seg = u0 % a.nseg;
+    for (int k = 0; k < nu; ++k) {
+      const uint32_t ok = mbar_wait_ns(full + st, par, limit);
+      if (!__all_sync(0xffffffffu, ok)) {
+        sflag = 1;
+        break;
       }
-      if (committed > 0) {
-        // completes once every MMA issued above has; waited for before TMEM is read or freed
-        umma_commit(&done);
-        if (!mbar_wait_ns(&done, 0, kDrainNs)) sflag = 1;
+      tc_fence_after();
+      const int steps = (min(a.xs, n - seg * a.xs) + 15) >> 4;
+      // descriptors are linear in the start address (16-byte units: one per position)
+      const uint32_t off = (uint32_t)(st * a.stage_bytes) >> 4;
+      const uint32_t a_lo = (uint32_t)a_base + off, b_lo = (uint32_t)b_base + off;
+#pragma unroll
+      for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+        for (int q = 0; q < DW_XS / 16; ++q)
+          if (q < steps)
+            umma_bf16_acc(leader, tmem + (uint32_t)(dx * DW_NC), a_lo + (uint32_t)(16 * q + dx), a_hi,
+                          b_lo + (uint32_t)(16 * q), b_hi, idesc);
+      umma_commit(leader, empty + st);
+      committed = k + 1;
+      if (++seg == a.nseg) seg = 0;
+      if (++st == S) {
+        st = 0;
+        par ^= 1;
       }
+    }
+    if (committed > 0) {
+      // completes once every MMA issued above has; waited for before TMEM is read or freed
+      umma_commit(leader, &done);
+      if (!mbar_wait_ns(&done, 0, kDrainNs)) sflag = 1;
     }
     __syncwarp();
   } else if (bias) {

@@ -38,19 +38,35 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16_mn(int M, int N) {
   return umma_idesc_bf16(M, N) | (1u << 15) | (1u << 16);
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+// One lane of the calling warp (all lanes call it; the same lane every time): 1 there, 0 on
+// the others. A warp issues its MMAs as a whole, predicated on this: the loop, the waits and
+// the descriptors then stay warp-uniform, which keeps them in the uniform registers that
+// tcgen05.mma takes (from inside a one-lane branch every operand is moved there first).
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(e));
+  return e;
 }
 
-// arrive once on the mbarrier when every tcgen05.mma issued so far by this thread is done
-__device__ __forceinline__ void umma_commit(uint64_t* mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(mbar))
-               : "memory");
+// D += A B issued by the elected lane; descriptors as their low words and common high words
+// (a start address moves within the low word)
+__device__ __forceinline__ void umma_bf16_acc(uint32_t leader, uint32_t d_tmem, uint32_t a_lo,
+                                              uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                              uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred e, p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 e, %0, 0;\n\t"
+      "setp.eq.u32 p, %1, %1;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%1], a, b, %6, p;\n\t}\n" ::"r"(leader),
+      "r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc));
+}
+
+// arrive once on the mbarrier when every tcgen05.mma issued so far by the elected lane is done
+__device__ __forceinline__ void umma_commit(uint32_t leader, uint64_t* mbar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %0, 0;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%1];\n\t}\n" ::"r"(leader),
+      "r"(smem_u32(mbar))
+      : "memory");
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
@@ -77,10 +93,13 @@ __device__ __forceinline__ uint32_t mbar_test(uint64_t* mbar, uint32_t parity) {
 
 // Wait for phase `parity` of the mbarrier for at most limit_ns nanoseconds of the global
 // timer (and at most 2^26 polls); returns 1 when the phase completed, 0 when the wait gave
-// up. limit_ns = 0: one non-blocking check only. Each poll may suspend the thread for up to
-// kSuspendNs until the phase completes, so a waiting warp does not spin on the issue slots
-// the working warps of its scheduler need. The timer is read only after a first poll has
-// run out (most waits end within it), so a wait gives up at most two polls after its limit.
+// up. limit_ns = 0: one non-blocking check only. Short waits spin on the non-blocking check
+// (waking a suspended thread takes about a microsecond, which the stages of a pipeline would
+// pay one after another); after kSpinPolls of them each poll may suspend the thread for up to
+// kSuspendNs until the phase completes, so a long wait does not spin on the issue slots the
+// working warps of its scheduler need. The timer is read only after a first such poll has run
+// out, so a wait gives up at most two polls after its limit.
+constexpr int kSpinPolls = 64;
 constexpr uint32_t kSuspendNs = 10000;
 __device__ __forceinline__ uint32_t mbar_poll(uint64_t* mbar, uint32_t parity) {
   uint32_t done;
@@ -95,6 +114,8 @@ __device__ __forceinline__ uint32_t mbar_poll(uint64_t* mbar, uint32_t parity) {
 __device__ __forceinline__ uint32_t mbar_wait_ns(uint64_t* mbar, uint32_t parity, uint64_t limit_ns) {
   if (mbar_test(mbar, parity)) return 1;
   if (limit_ns == 0) return 0;
+  for (int it = 0; it < kSpinPolls; ++it)
+    if (mbar_test(mbar, parity)) return 1;
   if (mbar_poll(mbar, parity)) return 1;
   const uint64_t t0 = global_ns();
   for (int it = 0; it < (1 << 26); ++it) {
