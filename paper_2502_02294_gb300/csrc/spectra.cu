@@ -19,12 +19,27 @@ __device__ __forceinline__ int mode_bin(int k2, float& root) {
   return b;
 }
 
+// (hi, lo) += v, v >= any size: error-free sum of float pairs
+__device__ __forceinline__ void pair_add(float v, float vlo, float& hi, float& lo) {
+  const float s = __fadd_rn(hi, v), t = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(vlo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(v, t))));
+  hi = s;
+}
+
+// Sum of the float pair over the lanes lane .. last (inclusive) of a contiguous run of lanes,
+// right for the first lane of each run (all lanes of the warp call it).
+__device__ __forceinline__ void run_sum(int lane, int last, float& hi, float& lo) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const float h = __shfl_down_sync(0xffffffffu, hi, d), l = __shfl_down_sync(0xffffffffu, lo, d);
+    if (lane + d <= last) pair_add(h, l, hi, lo);
+  }
+}
+
 // hi + lo += x y, the product exact (hi, lo: unevaluated float pair, error-free sums)
 __device__ __forceinline__ void dot2(float x, float y, float& hi, float& lo) {
-  const float p = __fmul_rn(x, y), e = __fmaf_rn(x, y, -p);
-  const float s = __fadd_rn(hi, p), t = __fsub_rn(s, hi);
-  lo = __fadd_rn(lo, __fadd_rn(e, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(p, t))));
-  hi = s;
+  const float p = __fmul_rn(x, y);
+  pair_add(p, __fmaf_rn(x, y, -p), hi, lo);
 }
 
 // Sums per bin 1 .. nbins: mode weight, weight |k|, and NP weighted powers (NP = 0: the weight
@@ -33,8 +48,10 @@ __device__ __forceinline__ void dot2(float x, float y, float& hi, float& lo) {
 // to four, of 8-byte loads coalesced along k_x), so the bin, |k| and the histogram updates are
 // paid once for all four. FP64 runs at 1/64 of the FP32 rate here, so the work per mode is in
 // float: the bin in integers, |k| as a float root plus its residual, the products exact in
-// float pairs; only the histograms are double. At 128^3, 64 bins, this took 80 us (108 us for
-// NP = 3) with one FP64 update of every sum per mode; now 21 us (32 us).
+// float pairs; only the histograms are double, updated once per run of lanes of one bin (|k|
+// grows along a row; a shared-memory double atomic is a compare-and-swap loop). At 128^3, 64
+// bins, this took 80 us (108 us for NP = 3) with one FP64 update of every sum per mode, 21 us
+// (32 us) with one per thread; now 10 us (16 us).
 template <int NP>
 __global__ void __launch_bounds__(512) spectrum_bin_kernel(const cufftComplex* __restrict__ a,
                                                            const cufftComplex* __restrict__ b, int n,
@@ -48,46 +65,70 @@ __global__ void __launch_bounds__(512) spectrum_bin_kernel(const cufftComplex* _
   __syncthreads();
   const unsigned nh = n / 2 + 1;  // 0 <= |k| <= n / 2 along every axis
   const unsigned total = nh * nh * nh;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  // whole warps stay in the loop for the warp-wide sums
+  for (unsigned i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < total;
+       i0 += gridDim.x * blockDim.x) {
+    const unsigned i = i0 + lane;
     const int kx = i % nh;
     const unsigned r = i / nh;
     const int ky = r % nh, kz = r / nh;
     float root;
     const int k2 = kx * kx + ky * ky + kz * kz;
-    const int bin = mode_bin(k2, root) - 1;
-    if (bin < 0 || bin >= nbins) continue;
+    int bin = i < total ? mode_bin(k2, root) - 1 : -1;
+    if (bin >= nbins) bin = -1;
     // k and -k are distinct modes except at 0 and, for even n, at the Nyquist index
     const bool two_y = ky != 0 && 2 * ky != n, two_z = kz != 0 && 2 * kz != n;
     const int wx = (kx == 0 || 2 * kx == n) ? 1 : 2;
     const int mult = wx << ((int)two_y + (int)two_z);
-    atomicAdd(cnt + bin, (unsigned)mult);
+    if (bin >= 0) atomicAdd(cnt + bin, (unsigned)mult);
     if (NP) {
       // |k| = root + (k2 - root^2) / (2 root) to 1e-14; mult is a power of two
-      const float fm = (float)mult;
-      const float corr = __fdividef(__fmaf_rn(-root, root, (float)k2), 2.0f * root);
-      atomicAdd(hist + bin, (double)(fm * root) + (double)(fm * corr));
+      float khi = 0.0f, klo = 0.0f;
       float hi[NP ? NP : 1], lo[NP ? NP : 1];
 #pragma unroll
       for (int q = 0; q < NP; ++q) hi[q] = lo[q] = 0.0f;
+      if (bin >= 0) {
+        const float fm = (float)mult;
+        khi = fm * root;
+        klo = fm * __fdividef(__fmaf_rn(-root, root, (float)k2), 2.0f * root);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        if (((c & 1) && !two_y) || ((c & 2) && !two_z)) continue;
-        const long long o =
-            ((long long)((c & 2) ? n - kz : kz) * n + ((c & 1) ? n - ky : ky)) * nh + kx;
-        const cufftComplex x = a[o], y = b[o];
-        if (NP == 3) {
-          dot2(x.x, x.x, hi[0], lo[0]);
-          dot2(x.y, x.y, hi[0], lo[0]);
-          dot2(y.x, y.x, hi[1], lo[1]);
-          dot2(y.y, y.y, hi[1], lo[1]);
+        for (int c = 0; c < 4; ++c) {
+          if (((c & 1) && !two_y) || ((c & 2) && !two_z)) continue;
+          const long long o =
+              ((long long)((c & 2) ? n - kz : kz) * n + ((c & 1) ? n - ky : ky)) * nh + kx;
+          const cufftComplex x = a[o], y = b[o];
+          if (NP == 3) {
+            dot2(x.x, x.x, hi[0], lo[0]);
+            dot2(x.y, x.y, hi[0], lo[0]);
+            dot2(y.x, y.x, hi[1], lo[1]);
+            dot2(y.y, y.y, hi[1], lo[1]);
+          }
+          dot2(x.x, y.x, hi[NP - 1], lo[NP - 1]);
+          dot2(x.y, y.y, hi[NP - 1], lo[NP - 1]);
         }
-        dot2(x.x, y.x, hi[NP - 1], lo[NP - 1]);
-        dot2(x.y, y.y, hi[NP - 1], lo[NP - 1]);
-      }
-      const float fw = (float)wx;
+        const float fw = (float)wx;
 #pragma unroll
-      for (int q = 0; q < NP; ++q)
-        atomicAdd(hist + (size_t)(1 + q) * nbins + bin, (double)(fw * hi[q]) + (double)(fw * lo[q]));
+        for (int q = 0; q < NP; ++q) {
+          hi[q] *= fw;
+          lo[q] *= fw;
+        }
+      }
+      // |k| grows along a row, so lanes of one bin are neighbours: one update per run of them
+      const int left = __shfl_up_sync(0xffffffffu, bin, 1);
+      const bool head = lane == 0 || left != bin;
+      const unsigned heads = __ballot_sync(0xffffffffu, head);
+      const unsigned after = lane == 31 ? 0u : heads >> (lane + 1);
+      const int last = after ? lane + __ffs(after) - 1 : 31;
+      run_sum(lane, last, khi, klo);
+#pragma unroll
+      for (int q = 0; q < NP; ++q) run_sum(lane, last, hi[q], lo[q]);
+      if (head && bin >= 0) {
+        atomicAdd(hist + bin, (double)khi + (double)klo);
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+          atomicAdd(hist + (size_t)(1 + q) * nbins + bin, (double)hi[q] + (double)lo[q]);
+      }
     }
   }
   __syncthreads();
