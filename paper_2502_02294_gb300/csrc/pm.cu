@@ -125,10 +125,32 @@ struct PIdx {
   bool ok;
 };
 
-// grid (cdiv(n^3, threads), B); lanes past the last particle get ok = false (and a lattice
-// site past the end, never used)
+// Lattice site of a thread. BT > 0: a block of BT threads covers a brick of lattice sites, 32
+// (n a multiple of 32) or 16 sites in x, 4 in z for BT = 512 and 2 below, the rest in y; grid
+// (bricks in x times y, bricks in z, B). The CIC corners of a brick lie on few node rows, so
+// its warps share them in L1. BT = 0: blocks of 128 consecutive sites, grid (cdiv(n^3, 128),
+// B). Lanes without a particle get ok = false (and a lattice site past the end, never used).
+// In both, neighbouring lanes hold neighbouring x sites.
+__host__ __device__ constexpr int brick_lz(int bt) { return bt >= 512 ? 2 : 1; }
+__host__ __device__ constexpr int brick_lt(int bt) { return bt >= 512 ? 9 : (bt >= 256 ? 8 : 7); }
+
+template <int BT>
 __device__ __forceinline__ PIdx particle_index(int n) {
   PIdx r;
+  if (BT > 0) {
+    constexpr int lz = brick_lz(BT), lt = brick_lt(BT);
+    const int lx = (n & 31) == 0 ? 5 : 4, ly = lt - lz - lx;
+    const int nbx = (n + (1 << lx) - 1) >> lx;
+    const int by = blockIdx.x / nbx, bx = blockIdx.x - by * nbx;
+    const int t = threadIdx.x;
+    r.b = blockIdx.z;
+    r.qx = (bx << lx) + (t & ((1 << lx) - 1));
+    r.qy = (by << ly) + ((t >> lx) & ((1 << ly) - 1));
+    r.qz = (blockIdx.y << lz) + (t >> (lt - lz));
+    r.ok = r.qx < n && r.qy < n && r.qz < n;
+    r.p = (r.qz * n + r.qy) * n + r.qx;
+    return r;
+  }
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned nn = (unsigned)n * (unsigned)n;
   r.b = blockIdx.y;
@@ -150,10 +172,35 @@ __device__ __forceinline__ PIdx particle_index(int n) {
   return r;
 }
 
-static inline dim3 particle_grid(int n, int threads, int B) {
-  return dim3((unsigned)cdiv((long long)n * n * n, threads), B);
+constexpr int kPT = 128;  // threads per block of consecutive sites
+
+// Threads per brick of the particle kernels that gain from them. Late in a 128^3 run (flow of
+// several cells) the kick adjoint takes 106 us with bricks of 256 (108 with 512, 132 with 128)
+// against 129 us with consecutive sites, the readout of three fields 40 us against 50. The
+// kick (54 us against 57-58), the deposit (29 against 31) and its adjoint (47, the same) keep
+// consecutive sites: their blocks reuse little across rows, and the finer order balances
+// better.
+constexpr int kBrickKickAdj = 256, kBrickInterp = 256;
+
+// Bricks where they give every SM two blocks or more; small grids keep the finer blocks.
+static inline bool use_bricks(int bt, int n, int B) {
+  return (long long)n * n * n * B >= 2ll * 152 * bt;
 }
-constexpr int kPT = 128;  // threads per particle block
+static inline dim3 particle_grid(int bt, int n, int B) {
+  if (bt == 0) return dim3((unsigned)cdiv((long long)n * n * n, kPT), B);
+  const int lx = n % 32 == 0 ? 5 : 4, lz = brick_lz(bt), ly = brick_lt(bt) - lz - lx;
+  return dim3(cdiv(n, 1 << lx) * cdiv(n, 1 << ly), cdiv(n, 1 << lz), B);
+}
+
+// launch of a particle kernel with bricks of BT threads or consecutive sites
+#define DH_LAUNCH_PARTICLES(kernel, BT, n, B, st, ...)                                          \
+  do {                                                                                          \
+    if (use_bricks(BT, n, B))                                                                   \
+      DH_CUDA_TRY((launch_pdl(kernel<BT>, particle_grid(BT, n, B), BT, 0, st, __VA_ARGS__)));   \
+    else                                                                                        \
+      DH_CUDA_TRY((launch_pdl(kernel<0>, particle_grid(0, n, B), kPT, 0, st, __VA_ARGS__)));    \
+    DH_LAUNCH_CHECK();                                                                          \
+  } while (0)
 
 __device__ __forceinline__ void cic_setup(const float* s, const PIdx& q, int N3, int n,
                                           float inv_dx, Cic& c) {
@@ -168,12 +215,17 @@ __device__ __forceinline__ int node(const Cic& c, int oz, int oy, int ox, int n)
 
 // ------------------------------------------------------------------ deposit
 // Fixed point: 2^31 units per unit weight, accumulated in 64-bit integers (deterministic).
-// Values below 2^31 units convert through 32-bit integers (the 64-bit conversions run on
-// the FP64 pipe, which is slow on this part).
+// The 64-bit conversions run on the FP64 pipe, which is slow on this part (converted
+// unconditionally and selected, they held that pipe at 89 % and the deposit at 34 us per
+// 128^3), so values of magnitude up to 2^31 units, every CIC weight among them, convert
+// through 32-bit integers, and the 64-bit conversion is volatile: reached by a branch only.
 __device__ __forceinline__ unsigned long long to_fix(float x) {
   const float y = x * kFix;
+  if (y >= 0.0f && y < 4294967040.0f) return (unsigned long long)__float2uint_rn(y);
   if (fabsf(y) < 2147483520.0f) return (unsigned long long)(long long)__float2int_rn(y);
-  return (unsigned long long)__float2ll_rn(y);
+  long long r;
+  asm volatile("cvt.rni.s64.f32 %0, %1;" : "=l"(r) : "f"(y));
+  return (unsigned long long)r;
 }
 
 __device__ __forceinline__ float from_fix(unsigned long long a) {
@@ -206,7 +258,7 @@ __global__ void deposit_kernel(const float* __restrict__ s, const float* __restr
                                int n, float inv_dx, unsigned long long* __restrict__ acc) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index(n);  // lanes past the last particle stay for the warp exchange
+  const PIdx q = particle_index<0>(n);  // lanes past the last particle stay for the warp exchange
   s += (size_t)q.b * 3 * N3;
   acc += (size_t)q.b * N3;
   Cic c;
@@ -237,11 +289,9 @@ __global__ void deposit_kernel(const float* __restrict__ s, const float* __restr
 
 // grid (cdiv(N3, 1024), B): four cells per thread, 16-byte vector accesses where N3 and the
 // instance's pointers allow (add may alias out: each cell is read before it is written).
-// ZERO: the accumulator is cleared behind the read (else the caller clears it before the
-// next deposit with a memset, which streams at the copy rate: the clearing stores here cost
-// more than the conversion itself)
-template <bool ZERO>
-__global__ void fix_to_float_kernel(unsigned long long* __restrict__ acc, SArg scale,
+// The caller clears the accumulator before each deposit with a memset, which streams at the
+// copy rate (clearing it here behind the read took 20 us per 128^3 against 7 us without).
+__global__ void fix_to_float_kernel(const unsigned long long* __restrict__ acc, SArg scale,
                                     const float* add, int add_stride, float offset, float* out,
                                     int N3) {
   pdl_enter();
@@ -249,7 +299,7 @@ __global__ void fix_to_float_kernel(unsigned long long* __restrict__ acc, SArg s
   const float sc = scale.at(b);
   const int i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (i0 >= N3) return;
-  unsigned long long* a = acc + (size_t)b * N3;
+  const unsigned long long* a = acc + (size_t)b * N3;
   float* o = out + (size_t)b * N3;
   const float* ad = add ? add + (size_t)b * add_stride : nullptr;
   const uintptr_t al = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(o) |
@@ -258,11 +308,6 @@ __global__ void fix_to_float_kernel(unsigned long long* __restrict__ acc, SArg s
     const ulonglong2 v0 = *reinterpret_cast<const ulonglong2*>(a + i0);
     const ulonglong2 v1 = *reinterpret_cast<const ulonglong2*>(a + i0 + 2);
     const float4 r = ad ? *reinterpret_cast<const float4*>(ad + i0) : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (ZERO) {
-      const ulonglong2 z = make_ulonglong2(0ull, 0ull);
-      *reinterpret_cast<ulonglong2*>(a + i0) = z;
-      *reinterpret_cast<ulonglong2*>(a + i0 + 2) = z;
-    }
     float4 w;
     w.x = sc * from_fix(v0.x) + r.x + offset;
     w.y = sc * from_fix(v0.y) + r.y + offset;
@@ -273,7 +318,6 @@ __global__ void fix_to_float_kernel(unsigned long long* __restrict__ acc, SArg s
     const int i1 = i0 + 4 < N3 ? i0 + 4 : N3;
     for (int i = i0; i < i1; ++i) {
       const float cnt = from_fix(a[i]);
-      if (ZERO) a[i] = 0ull;
       o[i] = sc * cnt + (ad ? ad[i] : 0.0f) + offset;
     }
   }
@@ -281,20 +325,17 @@ __global__ void fix_to_float_kernel(unsigned long long* __restrict__ acc, SArg s
 
 sim_status launch_deposit(const float* s, const float* values, int n, float inv_dx,
                           unsigned long long* acc, int B, cudaStream_t st) {
-  DH_CUDA_TRY((launch_pdl(deposit_kernel, particle_grid(n, kPT, B), kPT, 0, st, s, values, n, inv_dx, acc)));
+  DH_CUDA_TRY((launch_pdl(deposit_kernel, particle_grid(0, n, B), kPT, 0, st, s, values, n, inv_dx, acc)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
 }
 
-sim_status launch_fix_to_float(unsigned long long* acc, SArg scale, const float* add,
+sim_status launch_fix_to_float(const unsigned long long* acc, SArg scale, const float* add,
                                int add_stride, float offset, float* out, int n, int B,
-                               cudaStream_t st, bool zero_acc) {
+                               cudaStream_t st) {
   const int N3 = n * n * n;
-  const dim3 grid(cdiv(N3, 1024), B);
-  if (zero_acc)
-    DH_CUDA_TRY((launch_pdl(fix_to_float_kernel<true>, grid, 256, 0, st, acc, scale, add, add_stride, offset, out, N3)));
-  else
-    DH_CUDA_TRY((launch_pdl(fix_to_float_kernel<false>, grid, 256, 0, st, acc, scale, add, add_stride, offset, out, N3)));
+  DH_CUDA_TRY((launch_pdl(fix_to_float_kernel, dim3(cdiv(N3, 1024), B), 256, 0, st, acc, scale, add,
+                          add_stride, offset, out, N3)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
 }
@@ -403,11 +444,12 @@ sim_status launch_gravity_adjoint(const float* lam_g, float* lam_delta, cufftCom
 }
 
 // ------------------------------------------------------------------ readout, kick, drift
+template <int BT>
 __global__ void interp_kernel(const float* __restrict__ grid, int nf, int n, float inv_dx,
                               const float* __restrict__ s, float* __restrict__ out) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index(n);
+  const PIdx q = particle_index<BT>(n);
   if (!q.ok) return;
   grid += (size_t)q.b * nf * N3;
   s += (size_t)q.b * 3 * N3;
@@ -430,8 +472,7 @@ __global__ void interp_kernel(const float* __restrict__ grid, int nf, int n, flo
 
 sim_status launch_interp(const float* grid, int nf, int n, float inv_dx, const float* s,
                          float* out, int B, cudaStream_t st) {
-  DH_CUDA_TRY((launch_pdl(interp_kernel, particle_grid(n, kPT, B), kPT, 0, st, grid, nf, n, inv_dx, s, out)));
-  DH_LAUNCH_CHECK();
+  DH_LAUNCH_PARTICLES(interp_kernel, kBrickInterp, n, B, st, grid, nf, n, inv_dx, s, out);
   return SIM_OK;
 }
 
@@ -464,7 +505,7 @@ __global__ void __launch_bounds__(128, 16) kick_drift_kernel(const float* s, flo
                                   int n, float inv_dx) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index(n);
+  const PIdx q = particle_index<0>(n);
   if (!q.ok) return;
   const int i = q.p;
   const size_t o3 = (size_t)q.b * 3 * N3;
@@ -503,7 +544,7 @@ __global__ void __launch_bounds__(128, 16) kick_drift_kernel(const float* s, flo
 sim_status launch_kick_drift(const float* s, float* s_out, const float* p, float* p_out,
                              const float* g, SArg K, SArg dtau, const float* zhat, float* aux,
                              int n, float inv_dx, int B, cudaStream_t st) {
-  DH_CUDA_TRY((launch_pdl(kick_drift_kernel, particle_grid(n, kPT, B), kPT, 0, st, s, s_out, p,
+  DH_CUDA_TRY((launch_pdl(kick_drift_kernel, particle_grid(0, n, B), kPT, 0, st, s, s_out, p,
                           p_out, g, K, dtau, zhat, aux, n, inv_dx)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
@@ -542,6 +583,7 @@ sim_status launch_gas_kick(const float* in, float* out, const float* g, SArg K, 
 // Adjoint of kick_drift_kernel: the particle part and, when lam_gas is not NULL, the gas
 // kick of the cell with the same index at the pre-kick gas state gas_u (its force adjoint
 // goes to lam_g4 with a float4 atomic: other particles scatter into the node concurrently).
+template <int BT>
 __global__ void kick_drift_adj_kernel(const float* __restrict__ s0, const float* __restrict__ p0,
                                       const float* __restrict__ g, SArg Ka, SArg dtaua,
                                       float* __restrict__ lam_s, float* __restrict__ lam_p,
@@ -550,7 +592,7 @@ __global__ void kick_drift_adj_kernel(const float* __restrict__ s0, const float*
                                       int n, float inv_dx) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index(n);
+  const PIdx q = particle_index<BT>(n);
   const size_t o3 = (size_t)q.b * 3 * N3;
   s0 += o3;
   if (p0) p0 += o3;
@@ -673,8 +715,8 @@ sim_status launch_kick_drift_adjoint(const float* s0, const float* p0, const flo
                                      SArg dtau, float* lam_s, float* lam_p, float4* lam_g4,
                                      DPart dK, DPart ddtau, const float* gas_u, float* lam_gas,
                                      int n, float inv_dx, int B, cudaStream_t st) {
-  DH_CUDA_TRY((launch_pdl(kick_drift_adj_kernel, particle_grid(n, kPT, B), kPT, 0, st, s0, p0, g, K, dtau, lam_s, lam_p, lam_g4, dK, ddtau, gas_u, lam_gas, n, inv_dx)));
-  DH_LAUNCH_CHECK();
+  DH_LAUNCH_PARTICLES(kick_drift_adj_kernel, kBrickKickAdj, n, B, st, s0, p0, g, K, dtau, lam_s, lam_p, lam_g4, dK,
+                      ddtau, gas_u, lam_gas, n, inv_dx);
   return SIM_OK;
 }
 
@@ -684,7 +726,7 @@ __global__ void deposit_adj_kernel(const float* __restrict__ s, const float* __r
                                    long long rho_stride) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index(n);
+  const PIdx q = particle_index<0>(n);
   s += (size_t)q.b * 3 * N3;
   lam_s += (size_t)q.b * 3 * N3;
   ld += (size_t)q.b * N3;
@@ -718,7 +760,7 @@ __global__ void deposit_adj_kernel(const float* __restrict__ s, const float* __r
 sim_status launch_deposit_adjoint(const float* s, const float* lam_delta, SArg cm,
                                   float* lam_s, DPart dcm, int n, float inv_dx, int B,
                                   cudaStream_t st, float* lam_rho, long long rho_stride) {
-  DH_CUDA_TRY((launch_pdl(deposit_adj_kernel, particle_grid(n, kPT, B), kPT, 0, st, s, lam_delta,
+  DH_CUDA_TRY((launch_pdl(deposit_adj_kernel, particle_grid(0, n, B), kPT, 0, st, s, lam_delta,
                           cm, lam_s, dcm, n, inv_dx, lam_rho, rho_stride)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
