@@ -431,11 +431,14 @@ __device__ __forceinline__ void conv_epilogue(const ConvArgs& a, const float acc
 #pragma unroll
     for (int c = 0; c < 5; ++c) a.y[((size_t)b * 5 + c) * N3 + v] = acc[c] + bias[c];
   } else if (MODE == CONV_OUT_APPLY) {
+    // all five loads before the first store (the compiler cannot move a load above one: the
+    // five round trips one after another made this layer twice as long as the others)
+    float* g = a.gas + (size_t)b * 5 * N3 + v;
+    float u[5];
 #pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      float* g = a.gas + ((size_t)b * 5 + c) * N3 + v;
-      *g += a.scale.v[c] * (acc[c] + bias[c]);
-    }
+    for (int c = 0; c < 5; ++c) u[c] = __ldcg(g + c * N3);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) g[c * N3] = u[c] + a.scale.v[c] * (acc[c] + bias[c]);
   } else {  // CONV_BWD
     const float4* zp = reinterpret_cast<const float4*>(a.zprev + ((size_t)b * N3 + v) * CH);
     float d[16];
