@@ -120,8 +120,23 @@ enum { TAG_IC_NOISE = 0, TAG_SUBGRID = 1 };
 //   v = m_f / rho, P = (gamma-1)(eps - |m|^2/(2 rho)), c = |v| + sqrt(max(gamma P/rho, 0))
 //   F = (m_f, m_x v, m_y v, m_z v, (eps+P) v) + P e_f,  F^R = (cU + F)/2, F^L = (cU - F)/2.
 // Reciprocal and square root use the SFU approximations (about 1 ulp), far below the
-// float32 round-off that accumulates over a sweep.
-__device__ __forceinline__ float fast_rcp(float x) { return __fdividef(1.0f, x); }
+// float32 round-off that accumulates over a sweep. The flush-to-zero forms are one
+// instruction each; the others scale denormal operands up and down around it (24
+// reciprocals per cell pair of a sweep). They give the same bits for every normal operand,
+// and the operands are normal where the result is used: rho, the limiter's denominator
+// (where a b > 0 is representable, |a + b| > 3e-23) and gamma P / rho, for which a denormal
+// value counts as zero (a sound speed below 1.1e-19).
+constexpr float kMinNormal = 1.17549435e-38f;
+__device__ __forceinline__ float fast_rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float fast_rsqrt(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 
 __device__ __forceinline__ void split_flux(const float u[5], int f, float gam, float FR[5],
                                            float FL[5]) {
@@ -131,7 +146,7 @@ __device__ __forceinline__ void split_flux(const float u[5], int f, float gam, f
   const float m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
   const float P = (gam - 1.0f) * (u[4] - 0.5f * m2 * inv);
   const float cs2 = gam * P * inv;
-  const float c = fabsf(v) + (cs2 > 0.0f ? cs2 * rsqrtf(cs2) : 0.0f);
+  const float c = fabsf(v) + (cs2 >= kMinNormal ? cs2 * fast_rsqrt(cs2) : 0.0f);
   float F[5];
   F[0] = md;
   F[1] = u[1] * v;
@@ -158,7 +173,7 @@ __device__ __forceinline__ void split_flux_vjp(const float u[5], int f, float ga
   const float m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
   const float P = (gam - 1.0f) * (u[4] - 0.5f * m2 * inv);
   const float cs2 = gam * P * inv;
-  const float rcs = cs2 > 0.0f ? rsqrtf(cs2) : 0.0f;
+  const float rcs = cs2 >= kMinNormal ? fast_rsqrt(cs2) : 0.0f;
   const float cs = cs2 * rcs;
   const float c = fabsf(v) + cs;
   float sig[5], del[5];
@@ -187,7 +202,7 @@ __device__ __forceinline__ void split_flux_vjp(const float u[5], int f, float ga
   lv += del[4] * (u[4] + P);
   // c = |v| + cs, cs = sqrt(gam P / rho): dcs/dP = gam/(2 cs rho), dcs/drho = -cs/(2 rho)
   lv += lc * (float)((v > 0.0f) - (v < 0.0f));
-  if (cs2 > 0.0f) {
+  if (cs2 >= kMinNormal) {
     lP += lc * 0.5f * gam * rcs * inv;
     lrho -= lc * 0.5f * cs * inv;
   }
@@ -204,15 +219,15 @@ __device__ __forceinline__ void split_flux_vjp(const float u[5], int f, float ga
 }
 
 // Gravity half kick of one gas cell (Sec. 2.2): m += rho g K, eps += K m.g + K^2 rho |g|^2 / 2,
-// g the three force components at offsets 0, N3, 2 N3 from g. Every product and sum is
+// g the three force components. Every product and sum is
 // rounded on its own (no FMA contraction), so that the kick kernel and the sweeps that kick
 // their cells as they load them give the same bits.
-__device__ __forceinline__ void gas_kick_cell(float u[5], const float* g, long long N3, float K) {
+__device__ __forceinline__ void gas_kick_cell(float u[5], const float g[3], float K) {
   const float rho = u[0];
   float mg = 0.0f, g2 = 0.0f;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    const float gj = __ldg(g + j * N3);
+    const float gj = g[j];
     const float mj = u[1 + j];
     mg = __fadd_rn(mg, __fmul_rn(mj, gj));
     g2 = __fadd_rn(g2, __fmul_rn(gj, gj));
@@ -221,12 +236,17 @@ __device__ __forceinline__ void gas_kick_cell(float u[5], const float* g, long l
   const float de = __fadd_rn(__fmul_rn(K, mg), __fmul_rn(__fmul_rn(__fmul_rn(0.5f, K), K), __fmul_rn(rho, g2)));
   u[4] = __fadd_rn(u[4], de);
 }
+// the same with the force components at offsets 0, N3, 2 N3 from g
+__device__ __forceinline__ void gas_kick_cell(float u[5], const float* g, long long N3, float K) {
+  const float gj[3] = {__ldg(g), __ldg(g + N3), __ldg(g + 2 * N3)};
+  gas_kick_cell(u, gj, K);
+}
 
 // Gated harmonic-mean (van Leer) limiter 2 max(ab,0) / (a + b + copysign(eps, a+b)).
 __device__ __forceinline__ float vanleer(float a, float b, float eps) {
   const float ab = a * b;
   const float s = a + b;
-  return ab > 0.0f ? __fdividef(2.0f * ab, s + copysignf(eps, s)) : 0.0f;
+  return ab > 0.0f ? (2.0f * ab) * fast_rcp(s + copysignf(eps, s)) : 0.0f;
 }
 
 __device__ __forceinline__ void vanleer_grad(float a, float b, float eps, float& da,

@@ -66,6 +66,23 @@ template <> struct SweepCfg<0> { static constexpr int S = 64, W = 4, NT = 128, S
 template <> struct SweepCfg<1> { static constexpr int S = DH_TILE_S, W = 32, NT = 256, SA = 16, WA = 32, NTA = 256; };
 template <> struct SweepCfg<2> { static constexpr int S = DH_TILE_S, W = 32, NT = 256, SA = 16, WA = 32, NTA = 256; };
 
+// Asynchronous copies global -> shared of the marching kernels: each thread copies its own
+// next two cells while it works on the current one and reads back only what it copied itself
+// (no barrier), so the loads cost no registers while they are in flight.
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(uint32_t dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+// all but the newest committed group of this thread have landed
+__device__ __forceinline__ void cp_async_wait_prev() {
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
+}
+
 // packed FP32x2 arithmetic of sm_100+ (FADD2 / FMUL2 / FFMA2: one issue slot for two lanes)
 __device__ __forceinline__ float2 pk(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -325,8 +342,8 @@ __device__ __forceinline__ void split_flux2(const float2 u[5], int f, float gam,
   const float2 m2 = fma2(u[1], u[1], fma2(u[2], u[2], mul2(u[3], u[3])));
   const float2 P = mul2(pk(gam - 1.0f), fma2(mul2(m2, hinv), pk(-1.0f), u[4]));
   const float2 cs2 = mul2(mul2(P, inv), pk(gam));
-  const float csx = cs2.x > 0.0f ? cs2.x * rsqrtf(cs2.x) : 0.0f;
-  const float csy = cs2.y > 0.0f ? cs2.y * rsqrtf(cs2.y) : 0.0f;
+  const float csx = cs2.x >= kMinNormal ? cs2.x * fast_rsqrt(cs2.x) : 0.0f;
+  const float csy = cs2.y >= kMinNormal ? cs2.y * fast_rsqrt(cs2.y) : 0.0f;
   const float2 hc = fma2(make_float2(csx, csy), pk(0.5f), make_float2(fabsf(hv.x), fabsf(hv.y)));
   float2 hF[5];
   hF[0] = mul2(u[f], pk(0.5f));
@@ -346,6 +363,10 @@ __device__ __forceinline__ void split_flux2(const float2 u[5], int f, float gam,
 // w even), a segment of L output cells from s0 along the sweep axis. (An x sweep on pairs of
 // y rows measured 2.2x slower than the tile at 128^3 and 6.7x at 256^3: its loads touch 64
 // rows per warp and thrash L1.)
+// Bound by instruction issue and, at 12 warps per SM, by what a warp waits for. With the cells
+// in a shared-memory ring (no shifted register windows, loads two cells ahead), no limiters in
+// the ramp-up and one-instruction reciprocals, a 128^3 sweep went from 29.3 M to 19.8 M warp
+// instructions and from 43 to 29 us under ncu (256^3: 275 -> 195 us in a run).
 template <int AXIS, int MINB>
 __global__ void __launch_bounds__(128, MINB)
 sweep_march2_kernel(const float* __restrict__ uin, float* __restrict__ uout, int n, SArg nua,
@@ -362,73 +383,121 @@ sweep_march2_kernel(const float* __restrict__ uin, float* __restrict__ uout, int
   if (kick_g) kick_g += (size_t)b * 3 * N3;
   const float nu = nua.at(b), kK = kick_K.at(b);
   const float2 hnu = pk(0.5f * nu), mnu = pk(-nu);
-  float2 Ua[5], Ub[5], Uc[5];  // U_{j-3}, U_{j-2}, U_{j-1}
   float2 FRp[5], f1m[5];       // F^R_{j-1}, first-order face j-3/2
   float2 R1[5], R2[5];         // Fh^R_{j-3}, Fh^R_{j-2}
   float2 dRa[5], dRb[5];       // (Fh^R_{j-3} - Fh^R_{j-4}) / 2, (Fh^R_{j-2} - Fh^R_{j-3}) / 2
   float2 L1[5], dLa[5];        // Fh^L_{j-2}, (Fh^L_{j-2} - Fh^L_{j-3}) / 2
   float2 F2m[5];               // limited face (j-4)+1/2
 #pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    const float init = (k == 0 || k == 4) ? 1.0f : 0.0f;
-    Ua[k] = Ub[k] = Uc[k] = pk(init);
+  for (int k = 0; k < 5; ++k)
     FRp[k] = f1m[k] = R1[k] = R2[k] = dRa[k] = dRb[k] = L1[k] = dLa[k] = F2m[k] = pk(0.0f);
-  }
+  // The thread's cells j-3 .. j+2 in shared memory (slot: iteration mod 8): the next two on
+  // their way while the current one is worked on, the earlier ones read back where they are
+  // used instead of held and shifted in registers. The force of the next cells (for the kick)
+  // has four slots.
+  extern __shared__ float sm[];
+  float2(*buf)[5][128] = reinterpret_cast<float2(*)[5][128]>(sm);
+  float2(*bufg)[3][128] = reinterpret_cast<float2(*)[3][128]>(buf + 8);
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const uint32_t bufa = (uint32_t)__cvta_generic_to_shared(&buf[0][0][tid]);
+  const uint32_t bufga = (uint32_t)__cvta_generic_to_shared(&bufg[0][0][tid]);
+  constexpr uint32_t kField = 128 * sizeof(float2);
+  const long long step = AXIS == 1 ? n : (long long)n * n;  // cells between neighbours of a line
+  auto fetch = [&](long long o, int it) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) cp_async8(bufa + (uint32_t)((it & 7) * 5 + k) * kField, uin + k * N3 + o);
+    if (kick_g)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) cp_async8(bufga + (uint32_t)((it & 3) * 3 + k) * kField, kick_g + k * N3 + o);
+  };
   int j = wrap_periodic(s0 - 3, n);
+  long long o = goff<AXIS>(j, w, t, n);
+  auto advance = [&]() {
+    ++j;
+    o += step;
+    if (j == n) {
+      j = 0;
+      o -= n * step;
+    }
+  };
+  fetch(o, 0);
+  cp_async_commit();
+  advance();
+  fetch(o, 1);
+  cp_async_commit();
+  long long oo = goff<AXIS>(s0, w, t, n);  // output cell
 #pragma unroll 1
   for (int it = 0; it < L + 6; ++it) {
     float2 u[5];
-    const long long o = goff<AXIS>(j, w, t, n);
+    cp_async_wait_prev();
+    float2* cell = &buf[it & 7][0][tid];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) u[k] = __ldg(reinterpret_cast<const float2*>(uin + k * N3 + o));
+    for (int k = 0; k < 5; ++k) u[k] = cell[k * 128];
     if (kick_g) {
       // the step's opening gas kick of both columns, as the kick kernel does it
-      float a[5], c[5];
+      float a[5], c[5], ga[3], gc[3];
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         a[k] = u[k].x;
         c[k] = u[k].y;
       }
-      gas_kick_cell(a, kick_g + o, N3, kK);
-      gas_kick_cell(c, kick_g + o + 1, N3, kK);
 #pragma unroll
-      for (int k = 0; k < 5; ++k) u[k] = make_float2(a[k], c[k]);
+      for (int k = 0; k < 3; ++k) {
+        const float2 gk = bufg[it & 3][k][tid];
+        ga[k] = gk.x;
+        gc[k] = gk.y;
+      }
+      gas_kick_cell(a, ga, kK);
+      gas_kick_cell(c, gc, kK);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        u[k] = make_float2(a[k], c[k]);
+        cell[k * 128] = u[k];
+      }
     }
+    advance();
+    if (it + 2 < L + 6) fetch(o, it + 2);
+    cp_async_commit();
     float2 FR[5], FL[5];
     split_flux2(u, F, gam, FR, FL);
-    float2 f1[5], uh[5];
+    float2 uh[5];
+    const float2* prev = &buf[(it - 1) & 7][0][tid];  // cell j-1 (any slot at it = 0: not used)
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      f1[k] = sub2(FRp[k], FL[k]);                       // face j-1/2
-      uh[k] = fma2(hnu, sub2(f1m[k], f1[k]), Uc[k]);     // Uh_{j-1}
+      const float2 f1 = sub2(FRp[k], FL[k]);                       // face j-1/2
+      uh[k] = fma2(hnu, sub2(f1m[k], f1), prev[k * 128]);          // Uh_{j-1}
+      f1m[k] = f1;
+      FRp[k] = FR[k];
     }
-    float2 FRh[5], FLh[5];
+    float2 FRh[5], FLh[5], dLb[5];
     split_flux2(uh, F, gam, FRh, FLh);
-    const int jo = s0 + it - 6;  // output cell j-3 (unwrapped)
-    const bool store = it >= 6 && jo < n;
-    const long long oo = goff<AXIS>(jo < n ? jo : 0, w, t, n);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) dLb[k] = mul2(sub2(FLh[k], L1[k]), pk(0.5f));
+    // the first limited face a segment needs is s0 - 1/2, at it = 5: the ramp-up iterations
+    // before it skip the limiters, the larger half of the work
+    if (it >= 5) {
+      const bool store = it >= 6 && s0 + it - 6 < n;  // output cell j-3
+      const float2* out_cell = &buf[(it - 3) & 7][0][tid];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const float2 fr = add2(R1[k], vanleer2(dRa[k], dRb[k], eps));
+        const float2 fl = sub2(L1[k], vanleer2(dLa[k], dLb[k], eps));
+        const float2 F2 = sub2(fr, fl);                  // face (j-3)+1/2
+        if (store)
+          *reinterpret_cast<float2*>(uout + k * N3 + oo) = fma2(mnu, sub2(F2, F2m[k]), out_cell[k * 128]);
+        F2m[k] = F2;
+      }
+      if (it >= 6) oo += step;
+    }
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      const float2 dLb = mul2(sub2(FLh[k], L1[k]), pk(0.5f));
-      const float2 fr = add2(R1[k], vanleer2(dRa[k], dRb[k], eps));
-      const float2 fl = sub2(L1[k], vanleer2(dLa[k], dLb, eps));
-      const float2 F2 = sub2(fr, fl);                    // face (j-3)+1/2
-      if (store)
-        *reinterpret_cast<float2*>(uout + k * N3 + oo) = fma2(mnu, sub2(F2, F2m[k]), Ua[k]);
-      F2m[k] = F2;
       dRa[k] = dRb[k];
       dRb[k] = mul2(sub2(FRh[k], R2[k]), pk(0.5f));
       R1[k] = R2[k];
       R2[k] = FRh[k];
-      dLa[k] = dLb;
+      dLa[k] = dLb[k];
       L1[k] = FLh[k];
-      Ua[k] = Ub[k];
-      Ub[k] = Uc[k];
-      Uc[k] = u[k];
-      FRp[k] = FR[k];
-      f1m[k] = f1[k];
     }
-    j = (j + 1 == n) ? 0 : j + 1;
   }
 }
 
@@ -450,6 +519,35 @@ __device__ __forceinline__ void vanleer_vg2(float2 a, float2 b, float eps, float
   db = make_float2(gx ? dB.x : 0.0f, gy ? dB.y : 0.0f);
 }
 
+// split_flux with every rounding spelled out, for the marching adjoint's recomputation of the
+// forward stages: there the last bits decide which limiters are gated and the sign of a velocity
+// near zero, and which products the compiler contracts into FMAs depends on the code around.
+// (The pressure enters the momentum flux and the enthalpy unrounded.)
+template <int F>
+__device__ __forceinline__ void split_flux_fixed(const float u[5], float gam, float FR[5],
+                                                 float FL[5]) {
+  const float inv = fast_rcp(u[0]);
+  const float v = __fmul_rn(u[F], inv);
+  constexpr int A = F == 2 ? 2 : 1, B = F == 2 ? 1 : 2;
+  const float m2 = __fmaf_rn(u[3], u[3], __fmaf_rn(u[A], u[A], __fmul_rn(u[B], u[B])));
+  const float e = __fmaf_rn(-(0.5f * m2), inv, u[4]);  // internal energy density
+  const float g1 = gam - 1.0f;
+  const float cs2 = __fmul_rn(__fmul_rn(gam, __fmul_rn(g1, e)), inv);
+  const float c = __fadd_rn(fabsf(v), cs2 >= kMinNormal ? __fmul_rn(cs2, fast_rsqrt(cs2)) : 0.0f);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    float f;
+    if (k == 0)
+      f = u[F];
+    else if (k == 4)
+      f = __fmul_rn(__fmaf_rn(g1, e, u[4]), v);
+    else
+      f = k == F ? __fmaf_rn(g1, e, __fmul_rn(u[k], v)) : __fmul_rn(u[k], v);
+    FR[k] = 0.5f * __fmaf_rn(c, u[k], f);
+    FL[k] = 0.5f * __fmaf_rn(c, u[k], -f);
+  }
+}
+
 // ------------------------------------------------------------- adjoint, marching form
 // Pass 1: each thread streams one line segment [s0, s0 + L) plus a halo and produces
 // lamUh_j for its own cells. At load i it recomputes the forward stages for cell i-1
@@ -462,6 +560,10 @@ __device__ __forceinline__ void vanleer_vg2(float2 a, float2 b, float eps, float
 // D = lf dbL/2 (daR, dbR the limiter partials of the right-moving face flux, daL, dbL of
 // the left-moving one). Cell i-4 is then complete and lamUh_{i-4} = VJP(Uh_{i-4}).
 // d/dnu gathers sum_t F2_t lf_t / nu - sum_j lamUh_j dF1_j / 2.
+// Bound by instruction issue at 12 warps per SM (148 registers, 51 KB of shared memory per
+// block). Windows in shared memory, loads two cells ahead, the face block skipped in the
+// ramp-up: 52 M -> 40 M warp instructions and 73 -> 55 us per 128^3 call in a pass (four
+// blocks per SM at 128 registers: 65 us).
 template <int AXIS, int FC = 1 + AXIS>
 __global__ void __launch_bounds__(128, 3)
 sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ lout,
@@ -482,132 +584,163 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
   double* dnu = dnub.at(b);
   const float hnu = 0.5f * nu, inv_nu = 1.0f / nu;
   float Uc[5], FRp[5], f1m[5];          // U_{i-1}, F^R_{i-1}, face (i-3/2)
-  float R0[5], R1[5], R2[5];            // Fh^R_{i-4}, Fh^R_{i-3}, Fh^R_{i-2}
-  float L0[5], L1[5];                   // Fh^L_{i-3}, Fh^L_{i-2}
-  float H0[5], H1[5], H2[5];            // Uh_{i-4}, Uh_{i-3}, Uh_{i-2}
-  float D0[5], D1[5], D2[5];            // dF1_{i-4}, dF1_{i-3}, dF1_{i-2}
-  float M0[5], M1[5], M2[5];            // lam_out_{i-3}, lam_out_{i-2}, lam_out_{i-1}
+  float R1[5], R2[5], dR[5];            // Fh^R_{i-3}, Fh^R_{i-2}, (Fh^R_{i-3} - Fh^R_{i-4}) / 2
+  float L1[5], dL[5];                   // Fh^L_{i-2}, (Fh^L_{i-2} - Fh^L_{i-3}) / 2
   float aR0[5], aR1[5], aR2[5];         // lamFh^R accumulators of cells i-4, i-3, i-2
   float aL0[5], aL1[5], aL2[5], aL3[5]; // lamFh^L accumulators of cells i-4 .. i-1
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    const float init = (k == 0 || k == 4) ? 1.0f : 0.0f;
-    Uc[k] = H0[k] = H1[k] = H2[k] = init;
-    FRp[k] = f1m[k] = R0[k] = R1[k] = R2[k] = L0[k] = L1[k] = 0.0f;
-    D0[k] = D1[k] = D2[k] = M0[k] = M1[k] = M2[k] = 0.0f;
+    Uc[k] = (k == 0 || k == 4) ? 1.0f : 0.0f;
+    FRp[k] = f1m[k] = R1[k] = R2[k] = dR[k] = L1[k] = dL[k] = 0.0f;
     aR0[k] = aR1[k] = aR2[k] = aL0[k] = aL1[k] = aL2[k] = aL3[k] = 0.0f;
   }
   float dnu_acc = 0.0f;
-  // loads run from s0 - 5 to s0 + L + 3: cells s0 .. s0 + L - 1 complete at i = j + 4
+  // The thread's own cells in shared memory: the state and adjoint of the next two cells on
+  // their way while the current one is worked on (four slots for U, eight for lam_out, whose
+  // cells i-3 and i-2 are read back where they are used), and Uh and dF1 of the cells
+  // i-4 .. i-1 that wait for their adjoint to be complete. Held in registers, these windows
+  // spilled and took a move per value and iteration.
+  extern __shared__ float sm[];
+  float(*bu)[5][128] = reinterpret_cast<float(*)[5][128]>(sm);
+  float(*bl)[5][128] = bu + 4;
+  float(*bh)[10][128] = reinterpret_cast<float(*)[10][128]>(bl + 8);
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const uint32_t bua = (uint32_t)__cvta_generic_to_shared(&bu[0][0][tid]);
+  const uint32_t bla = (uint32_t)__cvta_generic_to_shared(&bl[0][0][tid]);
+  constexpr uint32_t kField = 128 * sizeof(float);
   const int ww = live ? w : 0;
-  int j = wrap_periodic(s0 - 5, n);
-  float un[5], ln[5];
-  {
-    const long long o = goff<AXIS>(j, ww, t3, n);
+  const long long step = AXIS == 0 ? 1 : (AXIS == 1 ? n : (long long)n * n);
+  auto fetch = [&](long long o, int it) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      un[k] = __ldg(uin + k * N3 + o);
-      ln[k] = __ldg(lout + k * N3 + o);
+      cp_async4(bua + (uint32_t)((it & 3) * 5 + k) * kField, uin + k * N3 + o);
+      cp_async4(bla + (uint32_t)((it & 7) * 5 + k) * kField, lout + k * N3 + o);
     }
-  }
+  };
+  // loads run from s0 - 4 to s0 + L + 3: cells s0 .. s0 + L - 1 complete at i = j + 4
+  int j = wrap_periodic(s0 - 4, n);
+  long long o = goff<AXIS>(j, ww, t3, n);
+  long long oc = goff<AXIS>(s0, ww, t3, n);  // the cell that completes
+  auto advance = [&]() {
+    ++j;
+    o += step;
+    if (j == n) {
+      j = 0;
+      o -= n * step;
+    }
+  };
+  fetch(o, 0);
+  cp_async_commit();
+  advance();
+  fetch(o, 1);
+  cp_async_commit();
   // unrolled by the windows' period: the three-deep register windows rotate by renaming
-  // instead of moves (measured 119 -> 114 us per call at 128^3 despite a few spilled words)
+  // instead of moves
 #pragma unroll 3
-  for (int it = 0; it < L + 9; ++it) {
-    float u[5], lo[5];
+  for (int it = 0; it < L + 8; ++it) {
+    float u[5];
+    cp_async_wait_prev();
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      u[k] = un[k];
-      lo[k] = ln[k];
-    }
-    const int jn = (j + 1 == n) ? 0 : j + 1;
-    if (it + 1 < L + 9) {
-      const long long on = goff<AXIS>(jn, ww, t3, n);
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        un[k] = __ldg(uin + k * N3 + on);
-        ln[k] = __ldg(lout + k * N3 + on);
-      }
-    }
+    for (int k = 0; k < 5; ++k) u[k] = bu[it & 3][k][tid];
+    advance();
+    if (it + 2 < L + 8) fetch(o, it + 2);
+    cp_async_commit();
     // forward stages for cell i-1
     float FR[5], FL[5];
-    split_flux(u, F, gam, FR, FL);
-    float f1[5], dF[5], uh[5];
+    split_flux_fixed<F>(u, gam, FR, FL);
+    float uh[5];
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      f1[k] = FRp[k] - FL[k];  // face i-1/2
-      dF[k] = f1[k] - f1m[k];  // dF1_{i-1}
-      uh[k] = Uc[k] - hnu * dF[k];
+      const float f1 = __fsub_rn(FRp[k], FL[k]);  // face i-1/2
+      const float dF = __fsub_rn(f1, f1m[k]);     // dF1_{i-1}
+      uh[k] = __fmaf_rn(-hnu, dF, Uc[k]);
+      bh[it & 3][k][tid] = uh[k];
+      bh[it & 3][5 + k][tid] = dF;
+      f1m[k] = f1;
+      FRp[k] = FR[k];
+      Uc[k] = u[k];
     }
-    float FRh[5], FLh[5];
-    split_flux(uh, F, gam, FRh, FLh);
+    float FRh[5], FLh[5], bR[5], bL[5];
+    split_flux_fixed<F>(uh, gam, FRh, FLh);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      bR[k] = 0.5f * __fsub_rn(R2[k], R1[k]);
+      bL[k] = 0.5f * __fsub_rn(FLh[k], L1[k]);
+    }
     // face t = i-3: R from Fh^R_{i-4..i-2}, L from Fh^L_{i-3..i-1}; lf_t from lam_out
     // face t = i-3 belongs to this segment's d/dnu sum when t is one of its cells: over a
     // periodic line sum_k -lam_out_k (F2_k - F2_{k-1}) = sum_t F2_t lf_t / nu
-    const int jt = s0 + it - 8;  // unwrapped index of face cell t (face t + 1/2)
+    const int jt = s0 + it - 7;  // unwrapped index of face cell t (face t + 1/2)
     const bool face_in = (jt >= s0) && (jt < s0 + L) && (jt < n);
-    // components (0, 1) and (2, 3) as FP32x2 pairs, component 4 alone: the same operations
-#pragma unroll
-    for (int k = 0; k < 4; k += 2) {
-      const float2 lf = mul2(pk(nu), sub2(make_float2(M1[k], M1[k + 1]), make_float2(M0[k], M0[k + 1])));
-      const float2 r0 = make_float2(R0[k], R0[k + 1]), r1 = make_float2(R1[k], R1[k + 1]);
-      const float2 r2 = make_float2(R2[k], R2[k + 1]);
-      const float2 l0 = make_float2(L0[k], L0[k + 1]), l1 = make_float2(L1[k], L1[k + 1]);
-      const float2 aR = mul2(pk(0.5f), sub2(r1, r0)), bR = mul2(pk(0.5f), sub2(r2, r1));
-      const float2 aL = mul2(pk(0.5f), sub2(l1, l0));
-      const float2 bL = mul2(pk(0.5f), sub2(make_float2(FLh[k], FLh[k + 1]), l1));
-      float2 pR, daR, dbR, pL, daL, dbL;
-      vanleer_vg2(aR, bR, eps, pR, daR, dbR);
-      vanleer_vg2(aL, bL, eps, pL, daL, dbL);
-      const float2 hl = mul2(pk(0.5f), lf);
-      const float2 A = mul2(hl, daR), B = mul2(hl, dbR), C = mul2(hl, daL), D = mul2(hl, dbL);
-      const float2 a0 = sub2(make_float2(aR0[k], aR0[k + 1]), A);
-      const float2 a1 = add2(make_float2(aR1[k], aR1[k + 1]), sub2(add2(lf, A), B));
-      const float2 a2 = add2(make_float2(aR2[k], aR2[k + 1]), B);
-      const float2 b1 = sub2(make_float2(aL1[k], aL1[k + 1]), C);
-      const float2 b2 = add2(make_float2(aL2[k], aL2[k + 1]), sub2(sub2(C, lf), D));
-      const float2 b3 = add2(make_float2(aL3[k], aL3[k + 1]), D);
-      aR0[k] = a0.x; aR0[k + 1] = a0.y;
-      aR1[k] = a1.x; aR1[k + 1] = a1.y;
-      aR2[k] = a2.x; aR2[k + 1] = a2.y;
-      aL1[k] = b1.x; aL1[k + 1] = b1.y;
-      aL2[k] = b2.x; aL2[k + 1] = b2.y;
-      aL3[k] = b3.x; aL3[k + 1] = b3.y;
-      // d/dnu part 1: faces of the segment's output cells (t in [s0-1, s0+L))
-      if (face_in) {
-        const float2 f2 = mul2(sub2(add2(r1, pR), sub2(l1, pL)), lf);
-        dnu_acc += (f2.x + f2.y) * inv_nu;
-      }
-    }
-    {
-      const int k = 4;
-      const float lf = nu * (M1[k] - M0[k]);  // nu (lam_out_{t+1} - lam_out_t), t = i-3
-      const float aR = 0.5f * (R1[k] - R0[k]), bR = 0.5f * (R2[k] - R1[k]);
-      const float aL = 0.5f * (L1[k] - L0[k]), bL = 0.5f * (FLh[k] - L1[k]);
-      float pR, daR, dbR, pL, daL, dbL;
-      vanleer_vg(aR, bR, eps, pR, daR, dbR);
-      vanleer_vg(aL, bL, eps, pL, daL, dbL);
-      const float A = 0.5f * lf * daR, B = 0.5f * lf * dbR;
-      const float C = 0.5f * lf * daL, D = 0.5f * lf * dbL;
-      aR0[k] -= A;
-      aR1[k] += lf + A - B;
-      aR2[k] += B;
-      aL1[k] -= C;
-      aL2[k] += -lf + C - D;
-      aL3[k] += D;
-      if (face_in) dnu_acc += ((R1[k] + pR) - (L1[k] - pL)) * lf * inv_nu;
-    }
-    // cell i-4 is complete
-    const int jc = s0 + it - 9;  // unwrapped index of cell i-4
-    if (it >= 9 && live && jc < n) {
-      float luh[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-      split_flux_vjp(H0, F, gam, aR0, aL0, luh);
-      const long long oc = goff<AXIS>(jc, w, t3, n);
+    // the first face that reaches a cell of the segment is t = s0 - 2, at it = 5: the ramp-up
+    // iterations before it skip the face block (the larger half of the work)
+    if (it >= 5) {
+      float M0[5], M1[5];  // lam_out_{i-3}, lam_out_{i-2}
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
-        luh_out[k * N3 + oc] = luh[k];
-        dnu_acc -= 0.5f * luh[k] * D0[k];
+        M0[k] = bl[(it - 3) & 7][k][tid];
+        M1[k] = bl[(it - 2) & 7][k][tid];
       }
+      // components (0, 1) and (2, 3) as FP32x2 pairs
+#pragma unroll
+      for (int k = 0; k < 4; k += 2) {
+        const float2 lf = mul2(pk(nu), sub2(make_float2(M1[k], M1[k + 1]), make_float2(M0[k], M0[k + 1])));
+        const float2 r1 = make_float2(R1[k], R1[k + 1]), l1 = make_float2(L1[k], L1[k + 1]);
+        float2 pR, daR, dbR, pL, daL, dbL;
+        vanleer_vg2(make_float2(dR[k], dR[k + 1]), make_float2(bR[k], bR[k + 1]), eps, pR, daR, dbR);
+        vanleer_vg2(make_float2(dL[k], dL[k + 1]), make_float2(bL[k], bL[k + 1]), eps, pL, daL, dbL);
+        const float2 hl = mul2(pk(0.5f), lf);
+        const float2 A = mul2(hl, daR), B = mul2(hl, dbR), C = mul2(hl, daL), D = mul2(hl, dbL);
+        const float2 a0 = sub2(make_float2(aR0[k], aR0[k + 1]), A);
+        const float2 a1 = add2(make_float2(aR1[k], aR1[k + 1]), sub2(add2(lf, A), B));
+        const float2 a2 = add2(make_float2(aR2[k], aR2[k + 1]), B);
+        const float2 b1 = sub2(make_float2(aL1[k], aL1[k + 1]), C);
+        const float2 b2 = add2(make_float2(aL2[k], aL2[k + 1]), sub2(sub2(C, lf), D));
+        const float2 b3 = add2(make_float2(aL3[k], aL3[k + 1]), D);
+        aR0[k] = a0.x; aR0[k + 1] = a0.y;
+        aR1[k] = a1.x; aR1[k + 1] = a1.y;
+        aR2[k] = a2.x; aR2[k + 1] = a2.y;
+        aL1[k] = b1.x; aL1[k + 1] = b1.y;
+        aL2[k] = b2.x; aL2[k + 1] = b2.y;
+        aL3[k] = b3.x; aL3[k + 1] = b3.y;
+        // d/dnu part 1: faces of the segment's output cells (t in [s0-1, s0+L))
+        if (face_in) {
+          const float2 f2 = mul2(sub2(add2(r1, pR), sub2(l1, pL)), lf);
+          dnu_acc += (f2.x + f2.y) * inv_nu;
+        }
+      }
+      {
+        // component 4: its right and left moving limiter as the pair
+        const int k = 4;
+        const float lf = nu * (M1[k] - M0[k]);  // nu (lam_out_{t+1} - lam_out_t), t = i-3
+        float2 p, da, db;
+        vanleer_vg2(make_float2(dR[k], dL[k]), make_float2(bR[k], bL[k]), eps, p, da, db);
+        const float2 hl = pk(0.5f * lf);
+        const float2 AC = mul2(hl, da), BD = mul2(hl, db);
+        aR0[k] -= AC.x;
+        aR1[k] += lf + AC.x - BD.x;
+        aR2[k] += BD.x;
+        aL1[k] -= AC.y;
+        aL2[k] += -lf + AC.y - BD.y;
+        aL3[k] += BD.y;
+        if (face_in) dnu_acc += ((R1[k] + p.x) - (L1[k] - p.y)) * lf * inv_nu;
+      }
+    }
+    // cell i-4 is complete
+    if (it >= 8) {
+      if (live && s0 + it - 8 < n) {
+        float luh[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, h[5];
+        const float* hc = &bh[(it - 3) & 3][0][tid];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) h[k] = hc[k * 128];
+        split_flux_vjp(h, F, gam, aR0, aL0, luh);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          luh_out[k * N3 + oc] = luh[k];
+          dnu_acc -= 0.5f * luh[k] * hc[(5 + k) * 128];
+        }
+      }
+      oc += step;
     }
     // shift the windows
 #pragma unroll
@@ -619,25 +752,12 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
       aL1[k] = aL2[k];
       aL2[k] = aL3[k];
       aL3[k] = 0.0f;
-      H0[k] = H1[k];
-      H1[k] = H2[k];
-      H2[k] = uh[k];
-      D0[k] = D1[k];
-      D1[k] = D2[k];
-      D2[k] = dF[k];
-      R0[k] = R1[k];
+      dR[k] = bR[k];
       R1[k] = R2[k];
       R2[k] = FRh[k];
-      L0[k] = L1[k];
+      dL[k] = bL[k];
       L1[k] = FLh[k];
-      M0[k] = M1[k];
-      M1[k] = M2[k];
-      M2[k] = lo[k];
-      Uc[k] = u[k];
-      FRp[k] = FR[k];
-      f1m[k] = f1[k];
     }
-    j = jn;
   }
   if (dnu) {
     if (!live) dnu_acc = 0.0f;
@@ -710,8 +830,8 @@ __device__ __forceinline__ void split_flux_vjp2(const float2 u[5], int f, float 
   const float2 hm2inv = mul2(mul2(m2, inv), pk(0.5f));
   const float2 P = mul2(pk(gam - 1.0f), sub2(u[4], hm2inv));
   const float2 cs2 = mul2(mul2(P, inv), pk(gam));
-  const float rx = cs2.x > 0.0f ? rsqrtf(cs2.x) : 0.0f;
-  const float ry = cs2.y > 0.0f ? rsqrtf(cs2.y) : 0.0f;
+  const float rx = cs2.x >= kMinNormal ? fast_rsqrt(cs2.x) : 0.0f;
+  const float ry = cs2.y >= kMinNormal ? fast_rsqrt(cs2.y) : 0.0f;
   const float2 rcs = make_float2(rx, ry);
   const float2 cs = mul2(cs2, rcs);
   const float2 c = add2(make_float2(fabsf(v.x), fabsf(v.y)), cs);
@@ -739,7 +859,7 @@ __device__ __forceinline__ void split_flux_vjp2(const float2 u[5], int f, float 
   lv = fma2(del[4], add2(u[4], P), lv);
   const float2 sgn = make_float2((float)((v.x > 0.0f) - (v.x < 0.0f)), (float)((v.y > 0.0f) - (v.y < 0.0f)));
   lv = fma2(lc, sgn, lv);
-  // where cs2 <= 0: rcs = 0 and cs = 0, so both terms below vanish, as in split_flux_vjp
+  // where cs2 is not a positive normal: rcs = 0 and cs = 0, so both terms below vanish, as in split_flux_vjp
   lP = fma2(mul2(lc, pk(0.5f * gam)), mul2(rcs, inv), lP);
   lrho = fma2(mul2(lc, pk(-0.5f)), mul2(cs, inv), lrho);
   const float2 gP = mul2(pk(gam - 1.0f), lP);
@@ -1013,9 +1133,12 @@ sweep_adj_kernel(const float* __restrict__ uin, const float* __restrict__ lout,
 
 // Kernel variants (SIM_SWEEP_*): the shared-memory tile, or the marching form with line
 // segments of 32 or 16 cells (y and z sweeps only: marching along x is not coalesced).
-// The default, measured on GB300 for one instance: the tile is fastest up to n ~ 128
-// (51 us at 128^3 for every axis); marching with segments of 32 wins for y/z on larger
-// grids (335 us vs 386 us at 256^3). The adjoint defaults to the marching pair for every
+// The default, measured on GB300 for one instance, y and z sweeps in a stream of sweeps: the
+// paired march from n = 96 on (n even; 17.0 us against 17.6 for the tile at 96^3, 25 against
+// 41 at 128^3, 112 against 185 at 200^3, 175 against 342 at 256^3), the tile below (7.3 us
+// against 8.1 at 64^3: a march is one long dependent chain per thread, which small grids wait
+// for). Odd grids take the tile up to n = 191 and the march on single lines above (297
+// against 342 us at 256). The adjoint defaults to the marching pair for every
 // axis: y/z directly (2.1x the tile at 256^3), x on x <-> y transposed copies (the x tile
 // takes ~320 us at 128^3 against ~170 us for a y/z pair), with segments fitted to whole
 // waves (at 128^3 three segments of 43 cells: every block resident at once, 140 us per
@@ -1024,6 +1147,7 @@ sweep_adj_kernel(const float* __restrict__ uin, const float* __restrict__ lout,
 static int pick_fwd(int axis, int n, int variant) {
   if (axis == 0) return SIM_SWEEP_TILE;
   if (variant != SIM_SWEEP_DEFAULT) return variant;
+  if (n % 2 == 0 && n >= 96) return SIM_SWEEP_PAIR;
   return n >= 192 ? SIM_SWEEP_MARCH32 : SIM_SWEEP_TILE;
 }
 
@@ -1045,12 +1169,21 @@ static dim3 line_grid(int lanes, int n, int B, dim3 blk, int segs) {
   return dim3(cdiv(lanes, blk.x), B * cdiv(n, blk.y), segs);
 }
 
+// Dynamic shared memory of the marching kernels (blocks of up to 128 threads).
+constexpr int kPairSmem = (8 * 5 + 4 * 3) * 128 * (int)sizeof(float2);
+constexpr int kAdjSmem = (4 * 5 + 8 * 5 + 4 * 10) * 128 * (int)sizeof(float);
+
+// Cost of a segment's ramp-up, in output cells: the pair's 6 extra iterations, 5 of them
+// without the limiters (about 0.4 of an iteration), and the adjoint's 8, 5 of them without
+// the face block.
+constexpr int kPairRamp = 3, kAdjRamp = 5;
+
 // Segment length of a marching kernel for an n^3 grid of B instances: the number k of
 // segments per line that minimises waves(k) x (n / k + halo), a wave being the blocks of
 // shape blk that stay resident on all SMs at the kernel's register use (each thread
 // streams its segment plus the halo once).
 template <class Kern>
-static int fit_segment(Kern kernel, int n, int B, int halo, int lanes, dim3 blk) {
+static int fit_segment(Kern kernel, int n, int B, int halo, int lanes, dim3 blk, int smem = 0) {
   const int block = (int)(blk.x * blk.y);
   // resident blocks on the current device, per kernel, block size and device
   static std::mutex mu;
@@ -1068,7 +1201,7 @@ static int fit_segment(Kern kernel, int n, int B, int halo, int lanes, dim3 blk)
     if (it == cache.end()) {
       int sms = 0, per_sm = 0;
       if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0) != cudaSuccess) {
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess) {
         cudaGetLastError();
         return 32;
       }
@@ -1081,7 +1214,7 @@ static int fit_segment(Kern kernel, int n, int B, int halo, int lanes, dim3 blk)
   int best = n, best_cost = 1 << 30;
   for (int k = 1; k <= n; ++k) {
     const int L = cdiv(n, k);
-    if (L < 8) break;
+    if (L < 4) break;
     const long long blocks = layer * cdiv(n, L);
     const long long waves = (blocks + resident - 1) / resident;
     const long long cost = waves * (L + halo);
@@ -1115,15 +1248,15 @@ static sim_status launch_march2_mb(const float* uin, float* uout, int n, SArg nu
                                    float eps, int B, cudaStream_t st, const float* kick_g,
                                    SArg kick_K) {
   const dim3 blk = line_block(n / 2, 128);
-  const int L = fit_segment(sweep_march2_kernel<AXIS, MINB>, n, B, 6, n / 2, blk);
-  DH_CUDA_TRY((launch_pdl(sweep_march2_kernel<AXIS, MINB>, line_grid(n / 2, n, B, blk, cdiv(n, L)), blk, 0, st, uin, uout, n, nu, gam, eps, L, kick_g, kick_K)));
+  const int L = fit_segment(sweep_march2_kernel<AXIS, MINB>, n, B, kPairRamp, n / 2, blk, kPairSmem);
+  DH_CUDA_TRY((launch_pdl(sweep_march2_kernel<AXIS, MINB>, line_grid(n / 2, n, B, blk, cdiv(n, L)), blk, kPairSmem, st, uin, uout, n, nu, gam, eps, L, kick_g, kick_K)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
 }
 
-// Three resident blocks per SM (the registers capped at 168, 12 warps per SM) measured
-// fastest: 47 us at 128^3 and 277 us at 256^3 per y or z sweep, against 58 / 347 us at two
-// blocks (206 registers) and 66 / 347 us at four (128 registers, spilling).
+// Three resident blocks per SM (registers capped at 168, 12 warps per SM) measured fastest:
+// 25 us at 128^3 and 163 us at 256^3 per y or z sweep in a stream of sweeps, 34 us against 45
+// at four blocks (128 registers, spilling) in a 128^3 inference pass.
 template <int AXIS>
 static sim_status launch_march2_t(const float* uin, float* uout, int n, SArg nu, float gam,
                                   float eps, int B, cudaStream_t st, const float* kick_g,
@@ -1261,7 +1394,7 @@ static sim_status launch_adj_march_t(const float* uin, const float* lout, float*
     return SIM_EINVAL;
   }
   const dim3 blk = line_block(n, 128);
-  DH_CUDA_TRY((launch_pdl(sweep_adj_march_kernel<AXIS>, line_grid(n, n, B, blk, cdiv(n, L)), blk, 0, st, uin, lout, scratch, n, nu, gam, eps, dnu, L)));
+  DH_CUDA_TRY((launch_pdl(sweep_adj_march_kernel<AXIS>, line_grid(n, n, B, blk, cdiv(n, L)), blk, kAdjSmem, st, uin, lout, scratch, n, nu, gam, eps, dnu, L)));
   DH_LAUNCH_CHECK();
   return launch_adj_final<AXIS, 1 + AXIS>(uin, lout, scratch, lin, n, nu, gam, B, st);
 }
@@ -1275,7 +1408,7 @@ static sim_status launch_adj_x_transposed(const float* uin, const float* lout, f
   float *ut = scratch, *lt = scratch + F5, *it = scratch + 2 * F5, *luh = scratch + 3 * F5;
   DH_TRY(launch_transpose_xy(uin, ut, 5 * B, lout, lt, 5 * B, n, st));
   const dim3 blk = line_block(n, 128);
-  DH_CUDA_TRY((launch_pdl(sweep_adj_march_kernel<1, 1>, line_grid(n, n, B, blk, cdiv(n, L)), blk, 0, st, ut, lt, luh, n, nu, gam, eps, dnu, L)));
+  DH_CUDA_TRY((launch_pdl(sweep_adj_march_kernel<1, 1>, line_grid(n, n, B, blk, cdiv(n, L)), blk, kAdjSmem, st, ut, lt, luh, n, nu, gam, eps, dnu, L)));
   DH_LAUNCH_CHECK();
   const uintptr_t al = reinterpret_cast<uintptr_t>(ut) | reinterpret_cast<uintptr_t>(lt) |
                        reinterpret_cast<uintptr_t>(luh);
@@ -1299,7 +1432,7 @@ static sim_status launch_sweep_adj_t(const float* uin, const float* lout, float*
   if (variant != SIM_SWEEP_TILE) {
     const int L = variant == SIM_SWEEP_MARCH_FIT
                       ? fit_segment(sweep_adj_march_kernel<AXIS == 0 ? 1 : AXIS, AXIS == 0 ? 1 : 1 + AXIS>,
-                                    n, B, 9, n, line_block(n, 128))
+                                    n, B, kAdjRamp, n, line_block(n, 128), kAdjSmem)
                       : segment_length(variant);
     if (AXIS == 0) {
       if (!scratch) {
@@ -1318,15 +1451,21 @@ static sim_status launch_sweep_adj_t(const float* uin, const float* lout, float*
   return SIM_OK;
 }
 
+template <class Kern>
+static sim_status set_smem(Kern kernel, size_t bytes) {
+  DH_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  return SIM_OK;
+}
+
 template <int AXIS>
 static sim_status set_sweep_attributes() {
   using C = SweepCfg<AXIS>;
-  DH_CUDA_TRY(cudaFuncSetAttribute(sweep_fwd_kernel<AXIS>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(15 * (C::S + 6) * C::W * sizeof(float))));
-  DH_CUDA_TRY(cudaFuncSetAttribute(sweep_adj_kernel<AXIS>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(20 * (C::SA + 10) * C::WA * sizeof(float))));
+  DH_TRY(set_smem(sweep_fwd_kernel<AXIS>, 15 * (C::S + 6) * C::W * sizeof(float)));
+  DH_TRY(set_smem(sweep_adj_kernel<AXIS>, 20 * (C::SA + 10) * C::WA * sizeof(float)));
+  // the marching forms (x runs the adjoint of axis 1 on transposed copies)
+  constexpr int A = AXIS == 0 ? 1 : AXIS, F = AXIS == 0 ? 1 : 1 + AXIS;
+  DH_TRY(set_smem(sweep_adj_march_kernel<A, F>, kAdjSmem));
+  if (AXIS != 0) DH_TRY(set_smem(sweep_march2_kernel<A, 3>, kPairSmem));
   return SIM_OK;
 }
 
