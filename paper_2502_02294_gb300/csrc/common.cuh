@@ -311,6 +311,27 @@ __device__ __forceinline__ void block_sum_atomic(float v, double* out) {
   }
 }
 
+// The same for K sums at once (out[k] may be NULL): one round of barriers for all of them,
+// each summed in the order of block_sum_atomic.
+template <int K>
+__device__ __forceinline__ void block_sums_atomic(const float (&v)[K], double* const (&out)[K]) {
+  __shared__ float red[K][32];
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  const int nw = (blockDim.x * blockDim.y * blockDim.z) >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const float s = warp_sum(v[k]);
+    if ((tid & 31) == 0) red[k][tid >> 5] = s;
+  }
+  __syncthreads();
+  // warp q sums k = q, q + warps, ...
+  for (int k = tid >> 5; k < K; k += nw) {
+    const int lane = tid & 31;
+    const float s = warp_sum(lane < nw ? red[k][lane] : 0.0f);
+    if (lane == 0 && s != 0.0f && out[k]) atomicAdd(out[k], (double)s);
+  }
+}
+
 // periodic wrap of an index known to lie within a few periods of [0, n)
 __device__ __forceinline__ int wrap_periodic(int i, int n) {
   while (i < 0) i += n;
