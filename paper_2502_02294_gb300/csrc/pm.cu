@@ -341,13 +341,27 @@ sim_status launch_fix_to_float(const unsigned long long* acc, SArg scale, const 
 }
 
 // ------------------------------------------------------------------ Green's function
+// Division of a 31-bit index by a launch constant: q = (umulhi(i, m) + i) >> l (Granlund and
+// Montgomery 1994, Fig. 4.1, for i < 2^31). The two runtime divisions of a mode's index were
+// half of the Green's function kernels' instructions (45.7 us at 256^3, 41.1 without).
+struct FastDiv {
+  uint32_t d, m, l;
+  __device__ __forceinline__ uint32_t div(uint32_t i) const { return (__umulhi(i, m) + i) >> l; }
+};
+static FastDiv fast_div(uint32_t d) {
+  FastDiv f{d, 0, 0};
+  while ((1ull << f.l) < d) ++f.l;
+  f.m = (uint32_t)(((1ull << 32) * ((1ull << f.l) - d)) / d + 1);
+  return f;
+}
+
 // half-complex index -> signed integer wavenumbers and Nyquist flags
-__device__ __forceinline__ void kindex(int i, int n, int nh, int& kx, int& ky, int& kz,
+__device__ __forceinline__ void kindex(int i, int n, FastDiv dh, FastDiv dn, int& kx, int& ky, int& kz,
                                        bool& nx, bool& ny, bool& nz) {
-  kx = i % nh;
-  const int r = i / nh;
-  ky = r % n;
-  kz = r / n;
+  const int r = (int)dh.div((uint32_t)i);
+  kx = i - r * (int)dh.d;
+  kz = (int)dn.div((uint32_t)r);
+  ky = r - kz * n;
   const bool even = (n % 2 == 0);
   nx = even && kx == n / 2;
   ny = even && ky == n / 2;
@@ -358,7 +372,7 @@ __device__ __forceinline__ void kindex(int i, int n, int nh, int& kx, int& ky, i
 
 // gk[j] = i kgrad_j (pref / k^2) dk / n^3   (j = x, y, z); grid (cdiv(NC, 256), B)
 __global__ void green_kernel(const cufftComplex* __restrict__ dk, cufftComplex* __restrict__ gk,
-                             int n, float kf, SArg pref_norm) {
+                             int n, float kf, SArg pref_norm, FastDiv dh, FastDiv dn) {
   pdl_enter();
   const int nh = n / 2 + 1;
   const int NC = n * n * nh;
@@ -369,7 +383,7 @@ __global__ void green_kernel(const cufftComplex* __restrict__ dk, cufftComplex* 
   gk += (size_t)b * 3 * NC;
   int kx, ky, kz;
   bool nx, ny, nz;
-  kindex(i, n, nh, kx, ky, kz, nx, ny, nz);
+  kindex(i, n, dh, dn, kx, ky, kz, nx, ny, nz);
   const float fx = kf * kx, fy = kf * ky, fz = kf * kz;
   const float k2 = fx * fx + fy * fy + fz * fz;
   const float G = (k2 > 0.0f) ? pref_norm.at(b) / k2 : 0.0f;
@@ -384,7 +398,7 @@ __global__ void green_kernel(const cufftComplex* __restrict__ dk, cufftComplex* 
 // Adjoint: Y = sum_j (-i kgrad_j)(pref / k^2) L_j / n^3 (the operator with the sign of the
 // gradient flipped; the Hermitian weights of the half spectrum cancel, see sim_gravity_adjoint)
 __global__ void green_adj_kernel(const cufftComplex* __restrict__ lk, cufftComplex* __restrict__ yk,
-                                 int n, float kf, SArg pref_norm) {
+                                 int n, float kf, SArg pref_norm, FastDiv dh, FastDiv dn) {
   pdl_enter();
   const int nh = n / 2 + 1;
   const int NC = n * n * nh;
@@ -395,7 +409,7 @@ __global__ void green_adj_kernel(const cufftComplex* __restrict__ lk, cufftCompl
   yk += (size_t)b * NC;
   int kx, ky, kz;
   bool nx, ny, nz;
-  kindex(i, n, nh, kx, ky, kz, nx, ny, nz);
+  kindex(i, n, dh, dn, kx, ky, kz, nx, ny, nz);
   const float fx = kf * kx, fy = kf * ky, fz = kf * kz;
   const float k2 = fx * fx + fy * fy + fz * fz;
   const float G = (k2 > 0.0f) ? pref_norm.at(b) / k2 : 0.0f;
@@ -420,7 +434,8 @@ sim_status launch_gravity(const float* delta, float* g, cufftComplex* dk, cufftC
   DH_TRY(plans.set_stream(st));
   DH_TRY(fft_exec_r2c(plans.r2c1, delta, dk));
   const float kf = (float)(2.0 * M_PI / box);
-  DH_CUDA_TRY((launch_pdl(green_kernel, dim3(cdiv(NC, 256), B), 256, 0, st, dk, gk, n, kf, pref_norm)));
+  DH_CUDA_TRY((launch_pdl(green_kernel, dim3(cdiv(NC, 256), B), 256, 0, st, dk, gk, n, kf, pref_norm,
+                          fast_div(n / 2 + 1), fast_div(n))));
   DH_LAUNCH_CHECK();
   DH_TRY(fft_exec_c2r(plans.c2r3, gk, g));
   return SIM_OK;
@@ -437,7 +452,8 @@ sim_status launch_gravity_adjoint(const float* lam_g, float* lam_delta, cufftCom
   DH_TRY(plans.set_stream(st));
   DH_TRY(fft_exec_r2c(plans.r2c3, lam_g, gk));
   const float kf = (float)(2.0 * M_PI / box);
-  DH_CUDA_TRY((launch_pdl(green_adj_kernel, dim3(cdiv(NC, 256), B), 256, 0, st, gk, dk, n, kf, pref_norm)));
+  DH_CUDA_TRY((launch_pdl(green_adj_kernel, dim3(cdiv(NC, 256), B), 256, 0, st, gk, dk, n, kf, pref_norm,
+                          fast_div(n / 2 + 1), fast_div(n))));
   DH_LAUNCH_CHECK();
   DH_TRY(fft_exec_c2r(plans.c2r1, dk, lam_delta));
   return SIM_OK;
@@ -720,7 +736,8 @@ sim_status launch_kick_drift_adjoint(const float* s0, const float* p0, const flo
   return SIM_OK;
 }
 
-__global__ void deposit_adj_kernel(const float* __restrict__ s, const float* __restrict__ ld,
+// 32 registers instead of 40 (2,048 resident threads per SM): 48.6 -> 42.2 us at 128^3
+__global__ void __launch_bounds__(128, 16) deposit_adj_kernel(const float* __restrict__ s, const float* __restrict__ ld,
                                    SArg cma, float* __restrict__ lam_s, DPart dcm, int n,
                                    float inv_dx, float* __restrict__ lam_rho,
                                    long long rho_stride) {
