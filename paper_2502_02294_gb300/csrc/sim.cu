@@ -429,6 +429,10 @@ static FFTPlans& ic_plans(sim_t* h) { return h->B == 1 ? h->plans : h->plans1; }
 static sim_status part_join(float* dst6, const float* s, const float* p, const sim_t* h,
                             cudaStream_t st) {
   const size_t w = 3 * h->N3 * sizeof(float);
+  if (h->B == 1) {  // plain copies: half the time of pitched ones of a single row
+    DH_TRY(dcopy(dst6, s, w, st));
+    return dcopy((char*)dst6 + w, p, w, st);
+  }
   DH_CUDA_TRY(cudaMemcpy2DAsync(dst6, 2 * w, s, w, w, h->B, cudaMemcpyDeviceToDevice, st));
   DH_CUDA_TRY(cudaMemcpy2DAsync((char*)dst6 + w, 2 * w, p, w, w, h->B,
                                 cudaMemcpyDeviceToDevice, st));
@@ -438,6 +442,10 @@ static sim_status part_join(float* dst6, const float* s, const float* p, const s
 static sim_status part_split(float* s, float* p, const float* src6, const sim_t* h,
                              cudaStream_t st) {
   const size_t w = 3 * h->N3 * sizeof(float);
+  if (h->B == 1) {
+    DH_TRY(dcopy(s, src6, w, st));
+    return dcopy(p, (const char*)src6 + w, w, st);
+  }
   DH_CUDA_TRY(cudaMemcpy2DAsync(s, w, src6, 2 * w, w, h->B, cudaMemcpyDeviceToDevice, st));
   DH_CUDA_TRY(cudaMemcpy2DAsync(p, w, (const char*)src6 + w, 2 * w, w, h->B,
                                 cudaMemcpyDeviceToDevice, st));
@@ -481,11 +489,12 @@ static sim_status record_diag(sim_t* h, int idx, const float* gas, const float* 
 // without a tape is; a recompute for the reverse pass (T set, primary false) has none of
 // these side effects.
 // Tnext (with T, when the next step records into the chained slot after T): the slot whose
-// p0 takes this step's kicked momenta.
+// p0 takes this step's kicked momenta. slot_filled: the slot's input state and force are in
+// place already (nothing is copied into it).
 static sim_status forward_step(sim_t* h, int i, float** gas, float** gas_tmp, float* s, float* p,
                                float* g, const TapeSlot* T, bool merged_in = false,
                                bool kick_out = true, bool primary = false,
-                               const TapeSlot* Tnext = nullptr) {
+                               const TapeSlot* Tnext = nullptr, bool slot_filled = false) {
   const sim_params& P = h->prm;
   const int B = h->B;
   cudaStream_t st = h->st;
@@ -499,7 +508,7 @@ static sim_status forward_step(sim_t* h, int i, float** gas, float** gas_tmp, fl
   // a chained slot (tape_slot): its input state, positions and force are the previous
   // slot's outputs, and its input momenta were written into its p0 by the previous step.
   const bool chained = T && merged_in;
-  if (T && !chained) {
+  if (T && !chained && !slot_filled) {
     DH_TRY(dcopy(T->U0, *gas, gb, st));
     DH_TRY(dcopy(T->s0, s, vb, st));
     DH_TRY(dcopy(T->p0, p, vb, st));
@@ -1550,11 +1559,13 @@ sim_status sim_step_adjoint(sim_t* h, float* adj_gas, float* adj_part, double* a
   auto run = [&]() -> sim_status {
     DH_TRY(dzero(h->dslots, 2 * (size_t)B * SL_N * sizeof(double), st));
     DH_TRY(dzero(h->dglob, (size_t)B * NG * sizeof(double), st));
-    // recompute the step from its input with the tape
-    DH_TRY(dcopy(h->w_gas, h->prev_gas, 5 * N3 * sizeof(float), st));
-    DH_TRY(part_split(h->w_s, h->w_p, h->prev_part, h, st));
-    DH_TRY(compute_force(h, h->w_s, h->w_gas, pn_at(h, i), h->w_g));
-    DH_TRY(forward_step(h, i, &h->w_gas, &h->w_gas2, h->w_s, h->w_p, h->w_g, &T));
+    // recompute the step from its input straight into the tape slot; its closing kick changes
+    // nothing that the reverse pass reads
+    DH_TRY(dcopy(T.U0, h->prev_gas, 5 * N3 * sizeof(float), st));
+    DH_TRY(part_split(T.s0, T.p0, h->prev_part, h, st));
+    DH_TRY(compute_force(h, T.s0, T.U0, pn_at(h, i), T.g0));
+    DH_TRY(forward_step(h, i, &h->w_gas, &h->w_gas2, h->w_s, h->w_p, h->w_g, &T, false, false, false,
+                        nullptr, true));
     // reverse
     DH_TRY(dcopy(h->lam_gas, adj_gas, 5 * N3 * sizeof(float), st));
     DH_TRY(part_split(h->lam_s, h->lam_p, adj_part, h, st));
