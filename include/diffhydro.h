@@ -166,7 +166,7 @@ int32_t sim_batch_size(const sim_t* h);
  * tile; MARCH32 / MARCH16: one thread marches a line segment of 32 / 16 cells; MARCH_FIT:
  * the same with the segment length that fits the launch to whole waves of resident blocks
  * (forward: y and z only, the forward x sweep then uses the tile; adjoint: every axis,
- * x on x <-> y transposed copies, two passes through a 5-field scratch); PAIR: below. */
+ * y and z in one pass, x in two on x <-> y transposed copies); PAIR: below. */
 enum {
   SIM_SWEEP_DEFAULT = 0,
   SIM_SWEEP_TILE = 1,

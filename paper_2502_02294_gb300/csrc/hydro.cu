@@ -560,14 +560,19 @@ __device__ __forceinline__ void split_flux_fixed(const float u[5], float gam, fl
 // D = lf dbL/2 (daR, dbR the limiter partials of the right-moving face flux, daL, dbL of
 // the left-moving one). Cell i-4 is then complete and lamUh_{i-4} = VJP(Uh_{i-4}).
 // d/dnu gathers sum_t F2_t lf_t / nu - sum_j lamUh_j dF1_j / 2.
-// Bound by instruction issue at 12 warps per SM (148 registers, 51 KB of shared memory per
-// block). Windows in shared memory, loads two cells ahead, the face block skipped in the
-// ramp-up: 52 M -> 40 M warp instructions and 73 -> 55 us per 128^3 call in a pass (four
-// blocks per SM at 128 registers: 65 us).
-template <int AXIS, int FC = 1 + AXIS>
+// FUSE (y and z): pass 2 in the same march. lamUh of the cells next to the segment is computed
+// too, and cell i-5 is finished when its neighbours' lamUh are in registers, so lamUh never
+// goes through memory. Without it (x, on transposed copies) lamUh is the output and pass 2
+// writes the untransposed result.
+// Bound by instruction issue at 12 warps per SM (148 registers, 167 with FUSE, 61 KB of shared
+// memory per block). Windows in shared memory, loads two cells ahead, the face block skipped in
+// the ramp-up: 52 M -> 40 M warp instructions and 73 -> 55 us per 128^3 call of pass 1 in a
+// pass (four blocks per SM at 128 registers: 65 us). Pass 2 fused: about 9 us less per y or z
+// call at 128^3 than 55 + 25 us, 154 -> 146 us for the three sweeps at 96^3.
+template <int AXIS, int FC, bool FUSE>
 __global__ void __launch_bounds__(128, 3)
 sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ lout,
-                       float* __restrict__ luh_out, int n, SArg nua, float gam, float eps,
+                       float* __restrict__ out, int n, SArg nua, float gam, float eps,
                        DPart dnub, int L) {
   pdl_enter();
   constexpr int F = FC;  // momentum component along the sweep
@@ -579,7 +584,7 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
   const long long N3 = (long long)n * n * n;
   uin += (size_t)b * 5 * N3;
   lout += (size_t)b * 5 * N3;
-  luh_out += (size_t)b * 5 * N3;
+  out += (size_t)b * 5 * N3;
   const float nu = nua.at(b);
   double* dnu = dnub.at(b);
   const float hnu = 0.5f * nu, inv_nu = 1.0f / nu;
@@ -596,13 +601,13 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
   }
   float dnu_acc = 0.0f;
   // The thread's own cells in shared memory: the state and adjoint of the next two cells on
-  // their way while the current one is worked on (four slots for U, eight for lam_out, whose
-  // cells i-3 and i-2 are read back where they are used), and Uh and dF1 of the cells
-  // i-4 .. i-1 that wait for their adjoint to be complete. Held in registers, these windows
+  // their way while the current one is worked on (eight slots: the cells i-3, i-2 and, for pass
+  // 2, i-5 are read back where they are used), and Uh and dF1 of the cells i-4 .. i-1 that
+  // wait for their adjoint to be complete. Held in registers, these windows
   // spilled and took a move per value and iteration.
   extern __shared__ float sm[];
   float(*bu)[5][128] = reinterpret_cast<float(*)[5][128]>(sm);
-  float(*bl)[5][128] = bu + 4;
+  float(*bl)[5][128] = bu + 8;
   float(*bh)[10][128] = reinterpret_cast<float(*)[10][128]>(bl + 8);
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   const uint32_t bua = (uint32_t)__cvta_generic_to_shared(&bu[0][0][tid]);
@@ -613,14 +618,20 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
   auto fetch = [&](long long o, int it) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      cp_async4(bua + (uint32_t)((it & 3) * 5 + k) * kField, uin + k * N3 + o);
+      cp_async4(bua + (uint32_t)((it & 7) * 5 + k) * kField, uin + k * N3 + o);
       cp_async4(bla + (uint32_t)((it & 7) * 5 + k) * kField, lout + k * N3 + o);
     }
   };
-  // loads run from s0 - 4 to s0 + L + 3: cells s0 .. s0 + L - 1 complete at i = j + 4
-  int j = wrap_periodic(s0 - 4, n);
+  // cells c0 .. c0 + C - 1 get their lamUh: the segment's own, with FUSE one more on each side;
+  // loads run from c0 - 4, and cell c is complete when c + 4 is in (it = c - c0 + 8)
+  constexpr int X = FUSE ? 1 : 0;
+  const int c0 = s0 - X, iters = L + 2 * X + 8;
+  int j = wrap_periodic(c0 - 4, n);
   long long o = goff<AXIS>(j, ww, t3, n);
-  long long oc = goff<AXIS>(s0, ww, t3, n);  // the cell that completes
+  long long oc = goff<AXIS>(s0, ww, t3, n);  // the next output cell
+  float h0[5], hm[5];  // FUSE: lamUh_{i-5}, lamUh_{i-6}
+#pragma unroll
+  for (int k = 0; k < 5; ++k) h0[k] = hm[k] = 0.0f;
   auto advance = [&]() {
     ++j;
     o += step;
@@ -637,13 +648,13 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
   // unrolled by the windows' period: the three-deep register windows rotate by renaming
   // instead of moves
 #pragma unroll 3
-  for (int it = 0; it < L + 8; ++it) {
+  for (int it = 0; it < iters; ++it) {
     float u[5];
     cp_async_wait_prev();
 #pragma unroll
-    for (int k = 0; k < 5; ++k) u[k] = bu[it & 3][k][tid];
+    for (int k = 0; k < 5; ++k) u[k] = bu[it & 7][k][tid];
     advance();
-    if (it + 2 < L + 8) fetch(o, it + 2);
+    if (it + 2 < iters) fetch(o, it + 2);
     cp_async_commit();
     // forward stages for cell i-1
     float FR[5], FL[5];
@@ -670,9 +681,9 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
     // face t = i-3: R from Fh^R_{i-4..i-2}, L from Fh^L_{i-3..i-1}; lf_t from lam_out
     // face t = i-3 belongs to this segment's d/dnu sum when t is one of its cells: over a
     // periodic line sum_k -lam_out_k (F2_k - F2_{k-1}) = sum_t F2_t lf_t / nu
-    const int jt = s0 + it - 7;  // unwrapped index of face cell t (face t + 1/2)
+    const int jt = c0 + it - 7;  // unwrapped index of face cell t (face t + 1/2)
     const bool face_in = (jt >= s0) && (jt < s0 + L) && (jt < n);
-    // the first face that reaches a cell of the segment is t = s0 - 2, at it = 5: the ramp-up
+    // the first face that reaches cell c0 is t = c0 - 2, at it = 5: the ramp-up
     // iterations before it skip the face block (the larger half of the work)
     if (it >= 5) {
       float M0[5], M1[5];  // lam_out_{i-3}, lam_out_{i-2}
@@ -728,19 +739,47 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
     }
     // cell i-4 is complete
     if (it >= 8) {
-      if (live && s0 + it - 8 < n) {
-        float luh[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, h[5];
-        const float* hc = &bh[(it - 3) & 3][0][tid];
+      const int jc = c0 + it - 8;  // unwrapped index of cell i-4
+      float luh[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, h[5];
+      const float* hc = &bh[(it - 3) & 3][0][tid];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) h[k] = hc[k * 128];
-        split_flux_vjp(h, F, gam, aR0, aL0, luh);
+      for (int k = 0; k < 5; ++k) h[k] = hc[k * 128];
+      split_flux_vjp(h, F, gam, aR0, aL0, luh);
+      if (jc >= s0 && jc < s0 + L && jc < n) {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) dnu_acc -= 0.5f * luh[k] * hc[(5 + k) * 128];
+      }
+      if (!FUSE) {
+        if (live && jc < n)
+#pragma unroll
+          for (int k = 0; k < 5; ++k) out[k * N3 + oc] = luh[k];
+        oc += step;
+      } else {
+        // pass 2 of cell i-5, whose neighbours' lamUh are in registers
+        if (it >= 10) {
+          if (live && jc - 1 < n) {
+            const float* uc = &bu[(it - 5) & 7][0][tid];
+            const float* lc = &bl[(it - 5) & 7][0][tid];
+            float u5[5], lR[5], lL[5], lu[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+              u5[k] = uc[k * 128];
+              lR[k] = hnu * (luh[k] - h0[k]);
+              lL[k] = -hnu * (h0[k] - hm[k]);
+              lu[k] = lc[k * 128] + h0[k];
+            }
+            split_flux_vjp(u5, F, gam, lR, lL, lu);
+#pragma unroll
+            for (int k = 0; k < 5; ++k) out[k * N3 + oc] = lu[k];
+          }
+          oc += step;
+        }
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
-          luh_out[k * N3 + oc] = luh[k];
-          dnu_acc -= 0.5f * luh[k] * hc[(5 + k) * 128];
+          hm[k] = h0[k];
+          h0[k] = luh[k];
         }
       }
-      oc += step;
     }
     // shift the windows
 #pragma unroll
@@ -765,15 +804,13 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
   }
 }
 
-// Pass 2: lam_in_k = lam_out_k + lamUh_k + VJP(U_k; nu/2 (lamUh_{k+1} - lamUh_k),
-// -nu/2 (lamUh_k - lamUh_{k-1})), one thread per cell.
-template <int AXIS, int FC = 1 + AXIS>
+// Pass 2 of the x adjoint on x <-> y transposed copies, odd n: lam_in_k = lam_out_k + lamUh_k
+// + VJP(U_k; nu/2 (lamUh_{k+1} - lamUh_k), -nu/2 (lamUh_k - lamUh_{k-1})), one thread per cell.
 __global__ void __launch_bounds__(256)
 sweep_adj_final_kernel(const float* __restrict__ uin, const float* __restrict__ lout,
                        const float* __restrict__ luh, float* __restrict__ lin, int n,
                        SArg nua, float gam) {
   pdl_enter();
-  constexpr int F = FC;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = blockIdx.z / n;  // instance
   const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z - b * n;
@@ -785,24 +822,8 @@ sweep_adj_final_kernel(const float* __restrict__ uin, const float* __restrict__ 
   lin += (size_t)b * 5 * N3;
   const float nu = nua.at(b);
   const long long o = ((long long)z * n + y) * n + x;
-  int cm, cp;  // neighbour offsets along the sweep axis (periodic)
-  long long om, op;
-  if (AXIS == 0) {
-    cm = x == 0 ? n - 1 : x - 1;
-    cp = x + 1 == n ? 0 : x + 1;
-    om = o - x + cm;
-    op = o - x + cp;
-  } else if (AXIS == 1) {
-    cm = y == 0 ? n - 1 : y - 1;
-    cp = y + 1 == n ? 0 : y + 1;
-    om = o + (long long)(cm - y) * n;
-    op = o + (long long)(cp - y) * n;
-  } else {
-    cm = z == 0 ? n - 1 : z - 1;
-    cp = z + 1 == n ? 0 : z + 1;
-    om = o + (long long)(cm - z) * n * n;
-    op = o + (long long)(cp - z) * n * n;
-  }
+  const long long om = o + (long long)((y == 0 ? n - 1 : y - 1) - y) * n;  // periodic neighbours
+  const long long op = o + (long long)((y + 1 == n ? 0 : y + 1) - y) * n;
   float u[5], lR[5], lL[5], lu[5];
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
@@ -814,7 +835,7 @@ sweep_adj_final_kernel(const float* __restrict__ uin, const float* __restrict__ 
     lL[k] = -0.5f * nu * (h0 - hm);
     lu[k] = __ldg(lout + k * N3 + o) + h0;
   }
-  split_flux_vjp(u, F, gam, lR, lL, lu);
+  split_flux_vjp(u, 1, gam, lR, lL, lu);
 #pragma unroll
   for (int k = 0; k < 5; ++k) lin[k * N3 + o] = lu[k];
 }
@@ -873,96 +894,67 @@ __device__ __forceinline__ void split_flux_vjp2(const float2 u[5], int f, float 
   lu[0] = add2(lu[0], lrho);
 }
 
-// lam_in of cells x, x + 1 of row (y, z) (one instance's arrays): lam_out + lamUh + the
-// flux-split VJP of U with the face adjoints from lamUh of the neighbours along the axis
-template <int AXIS, int F>
-__device__ __forceinline__ void adj_final2_cells(const float* __restrict__ uin,
-                                                 const float* __restrict__ lout,
-                                                 const float* __restrict__ luh, int n, int x,
-                                                 int y, int z, float nu, float gam,
-                                                 float2 lu[5]) {
-  const long long N3 = (long long)n * n * n;
-  const long long o = ((long long)z * n + y) * n + x;
-  long long om, op;  // neighbours along the sweep axis (y or z), periodic
-  if (AXIS == 1) {
-    om = o + (long long)((y == 0 ? n - 1 : y - 1) - y) * n;
-    op = o + (long long)((y + 1 == n ? 0 : y + 1) - y) * n;
-  } else {
-    om = o + (long long)((z == 0 ? n - 1 : z - 1) - z) * n * n;
-    op = o + (long long)((z + 1 == n ? 0 : z + 1) - z) * n * n;
-  }
-  const float2 hnu = pk(0.5f * nu), mhnu = pk(-0.5f * nu);
-  float2 u[5], lR[5], lL[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    u[k] = __ldg(reinterpret_cast<const float2*>(uin + k * N3 + o));
-    const float2 h0 = __ldg(reinterpret_cast<const float2*>(luh + k * N3 + o));
-    const float2 hm = __ldg(reinterpret_cast<const float2*>(luh + k * N3 + om));
-    const float2 hp = __ldg(reinterpret_cast<const float2*>(luh + k * N3 + op));
-    lR[k] = mul2(hnu, sub2(hp, h0));
-    lL[k] = mul2(mhnu, sub2(h0, hm));
-    lu[k] = add2(__ldg(reinterpret_cast<const float2*>(lout + k * N3 + o)), h0);
-  }
-  split_flux_vjp2(u, F, gam, lR, lL, lu);
-}
-
-// grid (cdiv(n / 2, blockDim.x), cdiv(n, blockDim.y), n B); thread: cells x = 2 t, 2 t + 1
-// of row (y, z). TOUT (the x axis run on x <-> y transposed copies): blocks of 16 x 32
-// threads cover 32 x 32 cells of a plane, and the result goes out through a shared-memory
-// tile in the untransposed layout, cell (z, y, x) of the copies to (z, x, y) of lin.
-template <int AXIS, int FC = 1 + AXIS, bool TOUT = false>
-__global__ void __launch_bounds__(TOUT ? 512 : 128)
+// Pass 2 of the x adjoint on x <-> y transposed copies, n even: cells x, x + 1 of row (y, z)
+// per thread, grid (cdiv(n, 32), cdiv(n, 32), n B), blocks of 16 x 32 threads covering 32 x 32
+// cells of a plane; the result goes out through a shared-memory tile in the untransposed layout,
+// cell (z, y, x) of the copies to (z, x, y) of lin.
+__global__ void __launch_bounds__(512)
 sweep_adj_final2_kernel(const float* __restrict__ uin, const float* __restrict__ lout,
                         const float* __restrict__ luh, float* __restrict__ lin, int n,
                         SArg nua, float gam) {
   pdl_enter();
-  constexpr int F = FC;
   const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int b = blockIdx.z / n;
   const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z - b * n;
   const long long N3 = (long long)n * n * n;
-  if (TOUT) {
-    __shared__ float tile[5][32][33];  // [field][x - x0][y - y0]
-    const int lx = 2 * threadIdx.x, ly = threadIdx.y;
-    if (x < n && y < n) {
-      float2 lu[5];
-      adj_final2_cells<AXIS, F>(uin + (size_t)b * 5 * N3, lout + (size_t)b * 5 * N3,
-                                luh + (size_t)b * 5 * N3, n, x, y, z, nua.at(b), gam, lu);
+  __shared__ float tile[5][32][33];  // [field][x - x0][y - y0]
+  const int lx = 2 * threadIdx.x, ly = threadIdx.y;
+  if (x < n && y < n) {
+    uin += (size_t)b * 5 * N3;
+    lout += (size_t)b * 5 * N3;
+    luh += (size_t)b * 5 * N3;
+    const float nu = nua.at(b);
+    const long long o = ((long long)z * n + y) * n + x;
+    const long long om = o + (long long)((y == 0 ? n - 1 : y - 1) - y) * n;  // periodic neighbours
+    const long long op = o + (long long)((y + 1 == n ? 0 : y + 1) - y) * n;
+    const float2 hnu = pk(0.5f * nu), mhnu = pk(-0.5f * nu);
+    float2 u[5], lR[5], lL[5], lu[5];
 #pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        tile[k][lx][ly] = lu[k].x;
-        tile[k][lx + 1][ly] = lu[k].y;
-      }
+    for (int k = 0; k < 5; ++k) {
+      u[k] = __ldg(reinterpret_cast<const float2*>(uin + k * N3 + o));
+      const float2 h0 = __ldg(reinterpret_cast<const float2*>(luh + k * N3 + o));
+      const float2 hm = __ldg(reinterpret_cast<const float2*>(luh + k * N3 + om));
+      const float2 hp = __ldg(reinterpret_cast<const float2*>(luh + k * N3 + op));
+      lR[k] = mul2(hnu, sub2(hp, h0));
+      lL[k] = mul2(mhnu, sub2(h0, hm));
+      lu[k] = add2(__ldg(reinterpret_cast<const float2*>(lout + k * N3 + o)), h0);
     }
-    __syncthreads();
-    const int x0 = 2 * blockIdx.x * blockDim.x, y0 = blockIdx.y * blockDim.y;
-    float* out = lin + (size_t)b * 5 * N3;
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    if ((n & 3) == 0 && (reinterpret_cast<uintptr_t>(lin) & 15) == 0) {
-      // rows of 32 outputs as eight float4 (y0 + c and n are multiples of 4)
-      for (int e = tid; e < 5 * 32 * 8; e += 512) {
-        const int k = e >> 8, r = (e >> 3) & 31, c = (e & 7) << 2;
-        if (x0 + r < n && y0 + c < n)
-          *reinterpret_cast<float4*>(out + k * N3 + ((long long)z * n + x0 + r) * n + y0 + c) =
-              make_float4(tile[k][r][c], tile[k][r][c + 1], tile[k][r][c + 2], tile[k][r][c + 3]);
-      }
-    } else {
-      for (int e = tid; e < 5 * 32 * 32; e += 512) {
-        const int k = e >> 10, r = (e >> 5) & 31, c = e & 31;
-        if (x0 + r < n && y0 + c < n)
-          out[k * N3 + ((long long)z * n + x0 + r) * n + y0 + c] = tile[k][r][c];
-      }
+    split_flux_vjp2(u, 1, gam, lR, lL, lu);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      tile[k][lx][ly] = lu[k].x;
+      tile[k][lx + 1][ly] = lu[k].y;
     }
-    return;
   }
-  if (x >= n || y >= n) return;
-  float2 lu[5];
-  adj_final2_cells<AXIS, F>(uin + (size_t)b * 5 * N3, lout + (size_t)b * 5 * N3,
-                            luh + (size_t)b * 5 * N3, n, x, y, z, nua.at(b), gam, lu);
-  lin += (size_t)b * 5 * N3;
-  const long long o = ((long long)z * n + y) * n + x;
-#pragma unroll
-  for (int k = 0; k < 5; ++k) *reinterpret_cast<float2*>(lin + k * N3 + o) = lu[k];
+  __syncthreads();
+  const int x0 = 2 * blockIdx.x * blockDim.x, y0 = blockIdx.y * blockDim.y;
+  float* out = lin + (size_t)b * 5 * N3;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  if ((n & 3) == 0 && (reinterpret_cast<uintptr_t>(lin) & 15) == 0) {
+    // rows of 32 outputs as eight float4 (y0 + c and n are multiples of 4)
+    for (int e = tid; e < 5 * 32 * 8; e += 512) {
+      const int k = e >> 8, r = (e >> 3) & 31, c = (e & 7) << 2;
+      if (x0 + r < n && y0 + c < n)
+        *reinterpret_cast<float4*>(out + k * N3 + ((long long)z * n + x0 + r) * n + y0 + c) =
+            make_float4(tile[k][r][c], tile[k][r][c + 1], tile[k][r][c + 2], tile[k][r][c + 3]);
+    }
+  } else {
+    for (int e = tid; e < 5 * 32 * 32; e += 512) {
+      const int k = e >> 10, r = (e >> 5) & 31, c = e & 31;
+      if (x0 + r < n && y0 + c < n)
+        out[k * N3 + ((long long)z * n + x0 + r) * n + y0 + c] = tile[k][r][c];
+    }
+  }
 }
 
 // ------------------------------------------------------------------------- adjoint
@@ -1157,11 +1149,14 @@ static int pick_adj(int axis, int variant) {
   return (variant != SIM_SWEEP_DEFAULT && variant != SIM_SWEEP_PAIR) ? variant : SIM_SWEEP_MARCH_FIT;
 }
 
-// Block of a line kernel (line_index): the x lanes (n, or n / 2 for two columns per lane)
-// in whole warps up to `threads`, and the rest of the block's threads as rows.
+// Block of a line kernel (line_index): 128, 64 or 32 lanes along x, whichever leaves the fewest
+// idle (the widest of equals), and the rest of the block's `threads` as rows, so that every
+// block is full (96 lanes in one row of a block left a quarter of its threads unused).
 static dim3 line_block(int lanes, int threads) {
-  const int tx = std::min(threads, 32 * cdiv(lanes, 32));
-  return dim3(tx, std::max(1, threads / tx));
+  int tx = std::min(threads, 128);
+  for (int t = tx / 2; t >= 32; t /= 2)
+    if (cdiv(lanes, t) * t < cdiv(lanes, tx) * tx) tx = t;
+  return dim3(tx, threads / tx);
 }
 
 // Grid of a line kernel over an n^3 grid of B instances with `segs` segments per line.
@@ -1171,12 +1166,12 @@ static dim3 line_grid(int lanes, int n, int B, dim3 blk, int segs) {
 
 // Dynamic shared memory of the marching kernels (blocks of up to 128 threads).
 constexpr int kPairSmem = (8 * 5 + 4 * 3) * 128 * (int)sizeof(float2);
-constexpr int kAdjSmem = (4 * 5 + 8 * 5 + 4 * 10) * 128 * (int)sizeof(float);
+constexpr int kAdjSmem = (8 * 5 + 8 * 5 + 4 * 10) * 128 * (int)sizeof(float);
 
 // Cost of a segment's ramp-up, in output cells: the pair's 6 extra iterations, 5 of them
-// without the limiters (about 0.4 of an iteration), and the adjoint's 8, 5 of them without
-// the face block.
-constexpr int kPairRamp = 3, kAdjRamp = 5;
+// without the limiters (about 0.4 of an iteration), and the adjoint's 8 (10 with pass 2), 5 of
+// them without the face block.
+constexpr int kPairRamp = 3, kAdjRamp = 5, kAdjFusedRamp = 7;
 
 // Segment length of a marching kernel for an n^3 grid of B instances: the number k of
 // segments per line that minimises waves(k) x (n / k + halo), a wave being the blocks of
@@ -1365,38 +1360,16 @@ static sim_status launch_transpose_xy(const float* in0, float* out0, int nf0, co
   return SIM_OK;
 }
 
-// Pass 2 of the marching adjoint: the paired packed form when n is even and the arrays are
-// 8-byte aligned, else one cell per thread.
-template <int AXIS, int FC>
-static sim_status launch_adj_final(const float* uin, const float* lout, const float* luh,
-                                   float* lin, int n, SArg nu, float gam, int B, cudaStream_t st) {
-  const uintptr_t al = reinterpret_cast<uintptr_t>(uin) | reinterpret_cast<uintptr_t>(lout) |
-                       reinterpret_cast<uintptr_t>(luh) | reinterpret_cast<uintptr_t>(lin);
-  if (AXIS != 0 && n % 2 == 0 && al % 8 == 0) {  // x runs as AXIS 1 on transposed copies
-    const dim3 blk = line_block(n / 2, 128);
-    const dim3 g(cdiv(n / 2, blk.x), cdiv(n, blk.y), n * B);
-    DH_CUDA_TRY((launch_pdl(sweep_adj_final2_kernel<AXIS, FC>, g, blk, 0, st, uin, lout, luh, lin, n, nu, gam)));
-  } else {
-    const dim3 blk = line_block(n, 256);
-    const dim3 g(cdiv(n, blk.x), cdiv(n, blk.y), n * B);
-    DH_CUDA_TRY((launch_pdl(sweep_adj_final_kernel<AXIS, FC>, g, blk, 0, st, uin, lout, luh, lin, n, nu, gam)));
-  }
-  DH_LAUNCH_CHECK();
-  return SIM_OK;
-}
-
+// The adjoint of a y or z sweep: one launch of the march with pass 2 fused.
 template <int AXIS>
 static sim_status launch_adj_march_t(const float* uin, const float* lout, float* lin, int n,
-                                     SArg nu, float gam, float eps, DPart dnu, float* scratch,
-                                     int B, int L, cudaStream_t st) {
-  if (!scratch) {
-    set_error("internal: marching sweep adjoint needs a 5 n^3 scratch buffer per instance");
-    return SIM_EINVAL;
-  }
+                                     SArg nu, float gam, float eps, DPart dnu, int B, int L,
+                                     cudaStream_t st) {
   const dim3 blk = line_block(n, 128);
-  DH_CUDA_TRY((launch_pdl(sweep_adj_march_kernel<AXIS>, line_grid(n, n, B, blk, cdiv(n, L)), blk, kAdjSmem, st, uin, lout, scratch, n, nu, gam, eps, dnu, L)));
+  DH_CUDA_TRY((launch_pdl(sweep_adj_march_kernel<AXIS, 1 + AXIS, true>, line_grid(n, n, B, blk, cdiv(n, L)),
+                          blk, kAdjSmem, st, uin, lout, lin, n, nu, gam, eps, dnu, L)));
   DH_LAUNCH_CHECK();
-  return launch_adj_final<AXIS, 1 + AXIS>(uin, lout, scratch, lin, n, nu, gam, B, st);
+  return SIM_OK;
 }
 
 // The x adjoint as the y-marching pair on x <-> y transposed copies (momentum component 1
@@ -1408,7 +1381,7 @@ static sim_status launch_adj_x_transposed(const float* uin, const float* lout, f
   float *ut = scratch, *lt = scratch + F5, *it = scratch + 2 * F5, *luh = scratch + 3 * F5;
   DH_TRY(launch_transpose_xy(uin, ut, 5 * B, lout, lt, 5 * B, n, st));
   const dim3 blk = line_block(n, 128);
-  DH_CUDA_TRY((launch_pdl(sweep_adj_march_kernel<1, 1>, line_grid(n, n, B, blk, cdiv(n, L)), blk, kAdjSmem, st, ut, lt, luh, n, nu, gam, eps, dnu, L)));
+  DH_CUDA_TRY((launch_pdl(sweep_adj_march_kernel<1, 1, false>, line_grid(n, n, B, blk, cdiv(n, L)), blk, kAdjSmem, st, ut, lt, luh, n, nu, gam, eps, dnu, L)));
   DH_LAUNCH_CHECK();
   const uintptr_t al = reinterpret_cast<uintptr_t>(ut) | reinterpret_cast<uintptr_t>(lt) |
                        reinterpret_cast<uintptr_t>(luh);
@@ -1416,11 +1389,15 @@ static sim_status launch_adj_x_transposed(const float* uin, const float* lout, f
     // the second pass writes lin in the untransposed layout itself
     const dim3 blk(16, 32);
     const dim3 g(cdiv(n / 2, 16), cdiv(n, 32), n * B);
-    DH_CUDA_TRY((launch_pdl(sweep_adj_final2_kernel<1, 1, true>, g, blk, 0, st, ut, lt, luh, lin, n, nu, gam)));
+    DH_CUDA_TRY((launch_pdl(sweep_adj_final2_kernel, g, blk, 0, st, ut, lt, luh, lin, n, nu, gam)));
     DH_LAUNCH_CHECK();
     return SIM_OK;
   }
-  DH_TRY((launch_adj_final<1, 1>(ut, lt, luh, it, n, nu, gam, B, st)));
+  // odd n (or arrays that are not 8-byte aligned): one cell per thread, then the way back
+  const dim3 fblk = line_block(n, 256);
+  DH_CUDA_TRY((launch_pdl(sweep_adj_final_kernel, dim3(cdiv(n, fblk.x), cdiv(n, fblk.y), n * B), fblk, 0,
+                          st, ut, lt, luh, it, n, nu, gam)));
+  DH_LAUNCH_CHECK();
   return launch_transpose_xy(it, lin, 5 * B, nullptr, nullptr, 0, n, st);
 }
 
@@ -1430,18 +1407,20 @@ static sim_status launch_sweep_adj_t(const float* uin, const float* lout, float*
                                      int B, int variant, cudaStream_t st) {
   using C = SweepCfg<AXIS>;
   if (variant != SIM_SWEEP_TILE) {
+    constexpr bool FUSE = AXIS != 0;
     const int L = variant == SIM_SWEEP_MARCH_FIT
-                      ? fit_segment(sweep_adj_march_kernel<AXIS == 0 ? 1 : AXIS, AXIS == 0 ? 1 : 1 + AXIS>,
-                                    n, B, kAdjRamp, n, line_block(n, 128), kAdjSmem)
+                      ? fit_segment(sweep_adj_march_kernel<FUSE ? AXIS : 1, FUSE ? 1 + AXIS : 1, FUSE>, n, B,
+                                    FUSE ? kAdjFusedRamp : kAdjRamp, n, line_block(n, 128), kAdjSmem)
                       : segment_length(variant);
-    if (AXIS == 0) {
+    if constexpr (AXIS == 0) {
       if (!scratch) {
         set_error("internal: the transposed x adjoint needs a 20 n^3 scratch buffer per instance");
         return SIM_EINVAL;
       }
       return launch_adj_x_transposed(uin, lout, lin, n, nu, gam, eps, dnu, scratch, B, L, st);
+    } else {
+      return launch_adj_march_t<AXIS>(uin, lout, lin, n, nu, gam, eps, dnu, B, L, st);
     }
-    return launch_adj_march_t<AXIS>(uin, lout, lin, n, nu, gam, eps, dnu, scratch, B, L, st);
   }
   constexpr int NC = (C::SA + 10) * C::WA;
   const size_t smem = 20 * NC * sizeof(float);
@@ -1464,7 +1443,7 @@ static sim_status set_sweep_attributes() {
   DH_TRY(set_smem(sweep_adj_kernel<AXIS>, 20 * (C::SA + 10) * C::WA * sizeof(float)));
   // the marching forms (x runs the adjoint of axis 1 on transposed copies)
   constexpr int A = AXIS == 0 ? 1 : AXIS, F = AXIS == 0 ? 1 : 1 + AXIS;
-  DH_TRY(set_smem(sweep_adj_march_kernel<A, F>, kAdjSmem));
+  DH_TRY(set_smem(sweep_adj_march_kernel<A, F, AXIS != 0>, kAdjSmem));
   if (AXIS != 0) DH_TRY(set_smem(sweep_march2_kernel<A, 3>, kPairSmem));
   return SIM_OK;
 }
@@ -1548,8 +1527,8 @@ extern "C" sim_status sim_sweep_adjoint(const float* u_in, const float* lam_out,
     return SIM_EINVAL;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  // the tile needs no scratch; the marching pairs 20 n^3 floats
-  const bool need = variant != SIM_SWEEP_TILE;
+  // only the x march needs scratch (its transposed copies): 20 n^3 floats
+  const bool need = axis == 0 && variant != SIM_SWEEP_TILE;
   float* scratch = nullptr;
   if (need) DH_CUDA_TRY(cudaMallocAsync((void**)&scratch, 20ull * n * n * n * sizeof(float), st));
   const sim_status r =
