@@ -57,14 +57,16 @@ __device__ __forceinline__ LineIdx line_index(int n, int wmul) {
   return r;
 }
 
-// tile shapes (forward / adjoint): x sweep 64 x 4 lines, y/z sweeps 32 x 32 and 16 x 32
+// Tile shapes (forward / adjoint): x sweep 64 x 4 lines, y/z sweeps 16 x 32. The forward threads
+// are chosen so that the tile and its halo are two full rounds of the block's warps (280 cells =
+// 5 + 4 warps, 704 cells = 2 x 11 warps): with 128 and 256 threads the warps had 3, 2, 2, 2 and
+// 3, ..., 2 rounds and waited for one another at every barrier. MB resident blocks per SM cap
+// the registers at 48 and 40. x / y: 36 / 42 -> 33 / 35 us at 128^3, 292 / 342 -> 259 / 280 us at
+// 256^3, 5.8 / 5.3 -> 3.9 / 4.2 us at 48^3.
 template <int AXIS> struct SweepCfg;
-template <> struct SweepCfg<0> { static constexpr int S = 64, W = 4, NT = 128, SA = 64, WA = 4, NTA = 128; };
-#ifndef DH_TILE_S
-#define DH_TILE_S 16
-#endif
-template <> struct SweepCfg<1> { static constexpr int S = DH_TILE_S, W = 32, NT = 256, SA = 16, WA = 32, NTA = 256; };
-template <> struct SweepCfg<2> { static constexpr int S = DH_TILE_S, W = 32, NT = 256, SA = 16, WA = 32, NTA = 256; };
+template <> struct SweepCfg<0> { static constexpr int S = 64, W = 4, NT = 160, MB = 8, SA = 64, WA = 4, NTA = 128; };
+template <> struct SweepCfg<1> { static constexpr int S = 16, W = 32, NT = 352, MB = 4, SA = 16, WA = 32, NTA = 256; };
+template <> struct SweepCfg<2> { static constexpr int S = 16, W = 32, NT = 352, MB = 4, SA = 16, WA = 32, NTA = 256; };
 
 // Asynchronous copies global -> shared of the marching kernels: each thread copies its own
 // next two cells while it works on the current one and reads back only what it copied itself
@@ -121,7 +123,7 @@ __device__ __forceinline__ float2 face_flux2(const float2* R, const float2* L, i
 // interleaved float pairs (one 8-byte access and one FP32x2 instruction for two components)
 // and component 4 alone: per array [pair 0: NC float2][pair 1: NC float2][component 4: NC].
 template <int AXIS>
-__global__ void __launch_bounds__(SweepCfg<AXIS>::NT, 2)
+__global__ void __launch_bounds__(SweepCfg<AXIS>::NT, SweepCfg<AXIS>::MB)
 sweep_fwd_kernel(const float* __restrict__ uin, float* __restrict__ uout, int n, SArg nua,
                  float gam, float eps, const float* __restrict__ kick_g, SArg kick_K) {
   pdl_enter();
@@ -1126,11 +1128,10 @@ sweep_adj_kernel(const float* __restrict__ uin, const float* __restrict__ lout,
 // Kernel variants (SIM_SWEEP_*): the shared-memory tile, or the marching form with line
 // segments of 32 or 16 cells (y and z sweeps only: marching along x is not coalesced).
 // The default, measured on GB300 for one instance, y and z sweeps in a stream of sweeps: the
-// paired march from n = 96 on (n even; 17.0 us against 17.6 for the tile at 96^3, 25 against
-// 41 at 128^3, 112 against 185 at 200^3, 175 against 342 at 256^3), the tile below (7.3 us
-// against 8.1 at 64^3: a march is one long dependent chain per thread, which small grids wait
-// for). Odd grids take the tile up to n = 191 and the march on single lines above (297
-// against 342 us at 256). The adjoint defaults to the marching pair for every
+// paired march above n = 96 (n even; 25 us against 35 for the tile at 128^3, 56 against 72 at
+// 160^3, 163 against 280 at 256^3), the tile up to it (16.1 us against 16.7 at 96^3, 6.4
+// against 9.4 at 64^3: a march is one long dependent chain per thread, which small grids wait
+// for). Odd grids take the tile (280 us at 256 against 297 for the march on single lines). The adjoint defaults to the marching pair for every
 // axis: y/z directly (2.1x the tile at 256^3), x on x <-> y transposed copies (the x tile
 // takes ~320 us at 128^3 against ~170 us for a y/z pair), with segments fitted to whole
 // waves (at 128^3 three segments of 43 cells: every block resident at once, 140 us per
@@ -1139,8 +1140,7 @@ sweep_adj_kernel(const float* __restrict__ uin, const float* __restrict__ lout,
 static int pick_fwd(int axis, int n, int variant) {
   if (axis == 0) return SIM_SWEEP_TILE;
   if (variant != SIM_SWEEP_DEFAULT) return variant;
-  if (n % 2 == 0 && n >= 96) return SIM_SWEEP_PAIR;
-  return n >= 192 ? SIM_SWEEP_MARCH32 : SIM_SWEEP_TILE;
+  return n % 2 == 0 && n > 96 ? SIM_SWEEP_PAIR : SIM_SWEEP_TILE;
 }
 
 static int pick_adj(int axis, int variant) {
