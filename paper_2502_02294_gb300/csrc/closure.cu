@@ -495,7 +495,9 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3_kernel(ConvArgs a) {
   const uint32_t sa0 = smem_u32(sa);
   const unsigned long long limit = a.wait_ns;
 
-  // setup: slack zeroed, weights staged, barriers, TMEM allocated and zeroed
+  // setup: slack zeroed, barriers, TMEM allocated and zeroed while the kernel before drains;
+  // then the weights (and everything else that it may have written)
+  pdl_launch_dependents();
   const int nslack = SLK_BEFORE + SLK_AFTER;
   for (int i = tid; i < ring * 2 * nslack; i += CONV_THREADS) {
     const int sp = i / nslack, k = i - sp * nslack;
@@ -503,8 +505,6 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3_kernel(ConvArgs a) {
     *reinterpret_cast<uint4*>(sa + (size_t)sp * a.slot_pos * 16 + (size_t)pos * 16) =
         make_uint4(0u, 0u, 0u, 0u);
   }
-  for (int i = tid; i < 9 * 1536 / 16; i += CONV_THREADS)
-    reinterpret_cast<uint4*>(sw)[i] = __ldg(reinterpret_cast<const uint4*>(a.w) + i);
   if (tid == 0) {
     for (int i = 0; i < nin; ++i) {
       mbar_init(full + i, 1);
@@ -520,6 +520,10 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3_kernel(ConvArgs a) {
   tc_fence_after();
   const uint32_t tmem = *tslot;
   tmem_zero(tmem, 0, a.ncols, w, CONV_THREADS / 128);
+  pdl_wait();
+  for (int i = tid; i < 9 * 1536 / 16; i += CONV_THREADS)
+    reinterpret_cast<uint4*>(sw)[i] = __ldg(reinterpret_cast<const uint4*>(a.w) + i);
+  fence_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -688,10 +692,10 @@ static sim_status launch_conv(int mode, ConvArgs a, int B, cudaStream_t st) {
   a.ncols = g.ncols;
   const dim3 grid(cdiv(a.n, g.L), cdiv(a.n, g.Zc), B);
   switch (mode) {
-    case CONV_HIDDEN: conv3_kernel<CONV_HIDDEN><<<grid, CONV_THREADS, g.smem, st>>>(a); break;
-    case CONV_OUT_Y: conv3_kernel<CONV_OUT_Y><<<grid, CONV_THREADS, g.smem, st>>>(a); break;
-    case CONV_OUT_APPLY: conv3_kernel<CONV_OUT_APPLY><<<grid, CONV_THREADS, g.smem, st>>>(a); break;
-    default: conv3_kernel<CONV_BWD><<<grid, CONV_THREADS, g.smem, st>>>(a); break;
+    case CONV_HIDDEN: DH_CUDA_TRY((launch_pdl(conv3_kernel<CONV_HIDDEN>, grid, CONV_THREADS, g.smem, st, a))); break;
+    case CONV_OUT_Y: DH_CUDA_TRY((launch_pdl(conv3_kernel<CONV_OUT_Y>, grid, CONV_THREADS, g.smem, st, a))); break;
+    case CONV_OUT_APPLY: DH_CUDA_TRY((launch_pdl(conv3_kernel<CONV_OUT_APPLY>, grid, CONV_THREADS, g.smem, st, a))); break;
+    default: DH_CUDA_TRY((launch_pdl(conv3_kernel<CONV_BWD>, grid, CONV_THREADS, g.smem, st, a))); break;
   }
   DH_LAUNCH_CHECK();
   return SIM_OK;
@@ -800,6 +804,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
   const uint32_t g_x0 = a.g_whole ? 16u : 0u;  // dz position x0 within its half-line
   const unsigned long long limit = a.wait_ns;
 
+  pdl_launch_dependents();
   // positions that no copy writes meet zero dz positions: they only have to be finite
   for (int i = tid; i < S * a.stage_bytes / 16; i += DW_THREADS)
     reinterpret_cast<uint4*>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -818,6 +823,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
   tc_fence_after();
   const uint32_t tmem = tslot;
   if (w < 4) tmem_zero(tmem, 0, 3 * DW_NC, w, 1);
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1063,7 +1069,7 @@ static sim_status launch_dw(const bf16* in, const bf16* dz, int n, int B, float*
   const dim3 grid(cdiv(a.units, a.per_cta), 3);
   // at least 116 KB so that no second CTA (of this kernel or a convolution) shares the SM
   const size_t bytes = std::max<size_t>({(size_t)a.stages * a.stage_bytes, (size_t)DW_RED, (size_t)116 * 1024});
-  conv_dw_kernel<<<grid, DW_THREADS, bytes, st>>>(a);
+  DH_CUDA_TRY((launch_pdl(conv_dw_kernel, grid, DW_THREADS, bytes, st, a)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
 }
@@ -1072,6 +1078,7 @@ static sim_status launch_dw(const bf16* in, const bf16* dz, int n, int B, float*
 // x[b][v][f] = bf16((gas[b][f][v] - mu_f) / sigma_f), f < 5; channels 5..15 are zero
 __global__ void closure_pack_kernel(const float* __restrict__ gas, F5 mu, F5 inv_sigma,
                                     bf16* __restrict__ x, long long N3, int n) {
+  pdl_enter();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int b = blockIdx.y;
   if (i >= N3) return;
@@ -1089,6 +1096,7 @@ __global__ void closure_loss_kernel(const float* __restrict__ y, const float* __
                                     const float* __restrict__ gtg, F5 inv_s, float norm,
                                     bf16* __restrict__ dz4, double* __restrict__ loss,
                                     long long N3, int n) {
+  pdl_enter();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int b = blockIdx.y;
   float acc = 0.0f;
@@ -1238,8 +1246,8 @@ static F5 f5(const float* v) {
 static sim_status closure_forward(sim_closure_s* c, const float* gas, int n, int B, int mode,
                                   float* gas_apply, bool keep, cudaStream_t st) {
   const long long N3 = (long long)n * n * n;
-  closure_pack_kernel<<<dim3(cdiv(N3, 256), B), 256, 0, st>>>(gas, f5(c->mu), f5(c->inv_sigma),
-                                                              c->x, N3, n);
+  DH_CUDA_TRY((launch_pdl(closure_pack_kernel, dim3(cdiv(N3, 256), B), 256, 0, st, gas, f5(c->mu),
+                          f5(c->inv_sigma), c->x, N3, n)));
   DH_LAUNCH_CHECK();
   bf16* acts[4] = {c->x, c->a1, c->a2, keep ? c->a3 : c->a1};
   float* zs[3] = {keep ? c->z1 : nullptr, keep ? c->z2 : nullptr, keep ? c->z3 : nullptr};
@@ -1278,8 +1286,8 @@ static sim_status closure_backprop(sim_closure_s* c, const float* gas, const flo
   F5 inv_s;
   for (int f = 0; f < 5; ++f) inv_s.v[f] = 1.0f / c->scale[f];
   const float norm = (float)(1.0 / (5.0 * (double)N3 * B));
-  closure_loss_kernel<<<dim3(cdiv(N3, 256), B), 256, 0, st>>>(c->y, gas, target, inv_s, norm,
-                                                              c->d1, c->loss, N3, n);
+  DH_CUDA_TRY((launch_pdl(closure_loss_kernel, dim3(cdiv(N3, 256), B), 256, 0, st, c->y, gas, target,
+                          inv_s, norm, c->d1, c->loss, N3, n)));
   DH_LAUNCH_CHECK();
   // layer l: input activation acts[l], pre-activation of layer l - 1: zs[l - 1]
   const bf16* acts[4] = {c->x, c->a1, c->a2, c->a3};
