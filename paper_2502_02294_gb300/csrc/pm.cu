@@ -254,8 +254,14 @@ __device__ __forceinline__ XPair xpair(int a0, int a1, bool ok) {
   return XPair{take, lane < 31 && ((tk >> (lane + 1)) & 1u)};
 }
 
-__global__ void deposit_kernel(const float* __restrict__ s, const float* __restrict__ vals,
-                               int n, float inv_dx, unsigned long long* __restrict__ acc) {
+// UNIT: every value is 1, so a corner's weight is at most 2^31 units and travels and converts as
+// one 32-bit word (a warp that holds a non-finite position takes the general conversion):
+// 212 -> 191 us at 256^3.
+template <bool UNIT>
+__global__ void __launch_bounds__(128, 16) deposit_kernel(const float* __restrict__ s,
+                                                          const float* __restrict__ vals, int n,
+                                                          float inv_dx,
+                                                          unsigned long long* __restrict__ acc) {
   pdl_enter();
   const int N3 = n * n * n;
   const PIdx q = particle_index<0>(n);  // lanes past the last particle stay for the warp exchange
@@ -265,21 +271,30 @@ __global__ void deposit_kernel(const float* __restrict__ s, const float* __restr
   float v = 0.0f;
   if (q.ok) {
     cic_setup(s, q, N3, n, inv_dx, c);
-    v = vals ? vals[(size_t)q.b * N3 + q.p] : 1.0f;
+    v = UNIT ? 1.0f : vals[(size_t)q.b * N3 + q.p];
   } else {
     c = Cic{{0, 0}, {0, 0}, {0, 0}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
   }
+  const bool words = UNIT && __all_sync(0xffffffffu, c.wx[1] + c.wy[1] + c.wz[1] >= 0.0f);
 #pragma unroll
   for (int oz = 0; oz < 2; ++oz)
 #pragma unroll
     for (int oy = 0; oy < 2; ++oy) {
       const int a0 = node(c, oz, oy, 0, n), a1 = node(c, oz, oy, 1, n);
       const float wyz = c.wz[oz] * c.wy[oy];
-      unsigned long long f0 = to_fix(wyz * c.wx[0] * v);
-      const unsigned long long f1 = to_fix(wyz * c.wx[1] * v);
       const XPair x = xpair(a0, a1, q.ok);
-      const unsigned long long fl = __shfl_up_sync(0xffffffffu, f1, 1);
-      if (x.take) f0 += fl;
+      unsigned long long f0, f1;
+      if (words) {
+        const unsigned u1 = __float2uint_rn(wyz * c.wx[1] * kFix);
+        const unsigned ul = __shfl_up_sync(0xffffffffu, u1, 1);
+        f0 = (unsigned long long)__float2uint_rn(wyz * c.wx[0] * kFix) + (x.take ? ul : 0u);
+        f1 = u1;
+      } else {
+        f0 = to_fix(wyz * c.wx[0] * v);
+        f1 = to_fix(wyz * c.wx[1] * v);
+        const unsigned long long fl = __shfl_up_sync(0xffffffffu, f1, 1);
+        if (x.take) f0 += fl;
+      }
       if (q.ok) {
         if (f0) atomicAdd(acc + a0, f0);
         if (!x.given && f1) atomicAdd(acc + a1, f1);
@@ -325,7 +340,11 @@ __global__ void fix_to_float_kernel(const unsigned long long* __restrict__ acc, 
 
 sim_status launch_deposit(const float* s, const float* values, int n, float inv_dx,
                           unsigned long long* acc, int B, cudaStream_t st) {
-  DH_CUDA_TRY((launch_pdl(deposit_kernel, particle_grid(0, n, B), kPT, 0, st, s, values, n, inv_dx, acc)));
+  const dim3 grid = particle_grid(0, n, B);
+  if (values)
+    DH_CUDA_TRY((launch_pdl(deposit_kernel<false>, grid, kPT, 0, st, s, values, n, inv_dx, acc)));
+  else
+    DH_CUDA_TRY((launch_pdl(deposit_kernel<true>, grid, kPT, 0, st, s, values, n, inv_dx, acc)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
 }
@@ -370,15 +389,28 @@ __device__ __forceinline__ void kindex(int i, int n, FastDiv dh, FastDiv dn, int
   if (kz > n / 2) kz -= n;
 }
 
-// gk[j] = i kgrad_j (pref / k^2) dk / n^3   (j = x, y, z); grid (cdiv(NC, 256), B)
+// gk[j] = i kgrad_j (pref / k^2) dk / n^3   (j = x, y, z); grid (cdiv(NC, 256), B).
+// acc (may be NULL): the deposit's accumulator, n^3 per instance, cleared for the next deposit (two
+// cells per mode), one launch fewer per step than a memset.
 __global__ void green_kernel(const cufftComplex* __restrict__ dk, cufftComplex* __restrict__ gk,
-                             int n, float kf, SArg pref_norm, FastDiv dh, FastDiv dn) {
+                             int n, float kf, SArg pref_norm, FastDiv dh, FastDiv dn,
+                             unsigned long long* __restrict__ acc) {
   pdl_enter();
   const int nh = n / 2 + 1;
   const int NC = n * n * nh;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = blockIdx.y;
   if (i >= NC) return;
+  if (acc) {
+    const int N3 = n * n * n;
+    unsigned long long* a = acc + (size_t)b * N3;
+    if ((N3 & 1) == 0) {  // 16-byte aligned pairs
+      if (2 * i < N3) *reinterpret_cast<ulonglong2*>(a + 2 * i) = make_ulonglong2(0ull, 0ull);
+    } else {
+      if (2 * i < N3) a[2 * i] = 0ull;
+      if (2 * i + 1 < N3) a[2 * i + 1] = 0ull;
+    }
+  }
   dk += (size_t)b * NC;
   gk += (size_t)b * 3 * NC;
   int kx, ky, kz;
@@ -425,7 +457,7 @@ float gravity_pref_norm(double pref, int n) { return (float)(pref / ((double)n *
 
 sim_status launch_gravity(const float* delta, float* g, cufftComplex* dk, cufftComplex* gk,
                           int n, double box, SArg pref_norm, int B, FFTPlans& plans,
-                          cudaStream_t st) {
+                          cudaStream_t st, unsigned long long* clear_acc) {
   if (plans.B != B) {
     set_error("internal: FFT plans for batch %d used with batch %d", plans.B, B);
     return SIM_EINVAL;
@@ -435,7 +467,7 @@ sim_status launch_gravity(const float* delta, float* g, cufftComplex* dk, cufftC
   DH_TRY(fft_exec_r2c(plans.r2c1, delta, dk));
   const float kf = (float)(2.0 * M_PI / box);
   DH_CUDA_TRY((launch_pdl(green_kernel, dim3(cdiv(NC, 256), B), 256, 0, st, dk, gk, n, kf, pref_norm,
-                          fast_div(n / 2 + 1), fast_div(n))));
+                          fast_div(n / 2 + 1), fast_div(n), clear_acc)));
   DH_LAUNCH_CHECK();
   DH_TRY(fft_exec_c2r(plans.c2r3, gk, g));
   return SIM_OK;

@@ -44,10 +44,11 @@ sim_status launch_fix_to_float(const unsigned long long* acc, SArg scale, const 
                                cudaStream_t st);
 // pref / n^3 in float, the normalisation the Green's function kernels take
 float gravity_pref_norm(double pref, int n);
-// g (3 n^3) from delta (n^3): r2c, Green's function * i k * pref / n^3, c2r x3
+// g (3 n^3) from delta (n^3): r2c, Green's function * i k * pref / n^3, c2r x3; clear_acc (may
+// be NULL, 16-byte aligned): a fixed-point grid (B n^3) that is set to zero on the way
 sim_status launch_gravity(const float* delta, float* g, cufftComplex* dk, cufftComplex* gk,
                           int n, double box, SArg pref_norm, int B, FFTPlans& plans,
-                          cudaStream_t st);
+                          cudaStream_t st, unsigned long long* clear_acc = nullptr);
 // lam_delta (n^3) = (d g / d delta)^T lam_g (3 n^3)
 sim_status launch_gravity_adjoint(const float* lam_g, float* lam_delta, cufftComplex* gk,
                                   cufftComplex* dk, int n, double box, SArg pref_norm, int B,

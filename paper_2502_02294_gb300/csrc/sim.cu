@@ -150,7 +150,8 @@ struct sim_s {
   float *gas = nullptr, *gas2 = nullptr, *s = nullptr, *p = nullptr, *g = nullptr;
   float *star = nullptr, *aux = nullptr, *zhat = nullptr, *delta = nullptr;
   uint32_t* events = nullptr;
-  unsigned long long* acc = nullptr;
+  unsigned long long* acc = nullptr;  // deposit accumulator, zero between calls
+  bool acc_dirty = false;
   cufftComplex* ck = nullptr;  // max(4 B, 5) NC complex scratch
   float *noise = nullptr, *f4 = nullptr;
   float *init_gas = nullptr, *init_part = nullptr;
@@ -457,16 +458,20 @@ static sim_status compute_force(sim_t* h, const float* s, const float* gas, SArg
   const int B = h->B;
   if (!h->prm.gravity_on) return dzero(g, 3 * B * h->N3 * sizeof(float), h->st);
   DH_TRY(timed(h, SIM_KT_DEPOSIT, [&] {
-    // the accumulator cleared by a memset ahead of the deposit, not by the conversion
-    DH_TRY(dzero(h->acc, (size_t)B * h->N3 * sizeof(unsigned long long), h->st));
+    // the accumulator is zero between calls (the Green's function kernel clears it); after a
+    // call that failed in between it may not be
+    if (h->acc_dirty) DH_TRY(dzero(h->acc, (size_t)B * h->N3 * sizeof(unsigned long long), h->st));
+    h->acc_dirty = true;
     DH_TRY(launch_deposit(s, nullptr, h->n, (float)h->inv_dx, h->acc, B, h->st));
     return launch_fix_to_float(h->acc, sarg(h->d_cm), gas, (int)(5 * h->N3), -1.0f, h->delta,
                                h->n, B, h->st);
   }));
-  return timed(h, SIM_KT_POISSON, [&] {
+  DH_TRY(timed(h, SIM_KT_POISSON, [&] {
     return launch_gravity(h->delta, g, h->ck, h->ck + B * h->NC, h->n, h->prm.box, pn, B,
-                          h->plans, h->st);
-  });
+                          h->plans, h->st, h->acc);
+  }));
+  h->acc_dirty = false;
+  return SIM_OK;
 }
 
 // Diagnostics record `idx` (the state after step idx - 1; idx 0 is the initial state).
