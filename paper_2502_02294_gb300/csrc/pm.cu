@@ -304,8 +304,10 @@ __global__ void __launch_bounds__(128, 16) deposit_kernel(const float* __restric
 
 // grid (cdiv(N3, 1024), B): four cells per thread, 16-byte vector accesses where N3 and the
 // instance's pointers allow (add may alias out: each cell is read before it is written).
-// The caller clears the accumulator before each deposit with a memset, which streams at the
-// copy rate (clearing it here behind the read took 20 us per 128^3 against 7 us without).
+// The accumulator is left as it is (clearing it here behind the read took 20 us per 128^3
+// against 7 us without): a simulation's is cleared for the next call by the Green's function
+// kernel, which is bound by its trigonometry and hides the stores, a single call's by a memset
+// before the deposit.
 __global__ void fix_to_float_kernel(const unsigned long long* __restrict__ acc, SArg scale,
                                     const float* add, int add_stride, float offset, float* out,
                                     int N3) {

@@ -151,7 +151,7 @@ struct sim_s {
   float *star = nullptr, *aux = nullptr, *zhat = nullptr, *delta = nullptr;
   uint32_t* events = nullptr;
   unsigned long long* acc = nullptr;  // deposit accumulator, zero between calls
-  bool acc_dirty = false;
+  bool acc_dirty = false;             // a call failed and its clearing could not be enqueued
   cufftComplex* ck = nullptr;  // max(4 B, 5) NC complex scratch
   float *noise = nullptr, *f4 = nullptr;
   float *init_gas = nullptr, *init_part = nullptr;
@@ -275,12 +275,25 @@ static void restore(sim_t* h, const HostState& s) {
   h->ckpt_step = s.ckpt_step;
 }
 
+// Clear the deposit accumulator on `st` if a failed call may have left sums in it. Graphs hold
+// no clearing of their own, so this runs before a replay or a capture. A clearing that is only
+// captured has not run yet, so it does not settle the flag.
+static sim_status settle_acc(sim_t* h, cudaStream_t st) {
+  if (!h->acc_dirty) return SIM_OK;
+  DH_TRY(dzero(h->acc, (size_t)h->B * h->N3 * sizeof(unsigned long long), st));
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  DH_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
+  if (cs == cudaStreamCaptureStatusNone) h->acc_dirty = false;
+  return SIM_OK;
+}
+
 // Run `body` directly, or (graphs on) replay the graph captured for (kind, key) from the
 // same host state, capturing it first if there is none.
 template <class Body>
 static sim_status run_maybe_graph(sim_t* h, int kind, const std::vector<uintptr_t>& key,
                                   Body body) {
   if (!h->graphs || h->kt_on) return body();
+  DH_TRY(settle_acc(h, h->st));
   const HostState before = snapshot(h);
   for (GraphEntry& e : h->graph_cache) {
     if (e.kind == kind && e.key == key && e.before == before) {
@@ -457,21 +470,22 @@ static sim_status part_split(float* s, float* p, const float* src6, const sim_t*
 static sim_status compute_force(sim_t* h, const float* s, const float* gas, SArg pn, float* g) {
   const int B = h->B;
   if (!h->prm.gravity_on) return dzero(g, 3 * B * h->N3 * sizeof(float), h->st);
-  DH_TRY(timed(h, SIM_KT_DEPOSIT, [&] {
-    // the accumulator is zero between calls (the Green's function kernel clears it); after a
-    // call that failed in between it may not be
-    if (h->acc_dirty) DH_TRY(dzero(h->acc, (size_t)B * h->N3 * sizeof(unsigned long long), h->st));
-    h->acc_dirty = true;
+  DH_TRY(settle_acc(h, h->st));
+  sim_status r = timed(h, SIM_KT_DEPOSIT, [&] {
     DH_TRY(launch_deposit(s, nullptr, h->n, (float)h->inv_dx, h->acc, B, h->st));
     return launch_fix_to_float(h->acc, sarg(h->d_cm), gas, (int)(5 * h->N3), -1.0f, h->delta,
                                h->n, B, h->st);
-  }));
-  DH_TRY(timed(h, SIM_KT_POISSON, [&] {
-    return launch_gravity(h->delta, g, h->ck, h->ck + B * h->NC, h->n, h->prm.box, pn, B,
-                          h->plans, h->st, h->acc);
-  }));
-  h->acc_dirty = false;
-  return SIM_OK;
+  });
+  // the Green's function kernel clears the accumulator for the next call
+  if (r == SIM_OK)
+    r = timed(h, SIM_KT_POISSON, [&] {
+      return launch_gravity(h->delta, g, h->ck, h->ck + B * h->NC, h->n, h->prm.box, pn, B,
+                            h->plans, h->st, h->acc);
+    });
+  if (r != SIM_OK)  // the kernel that clears may not have been launched
+    h->acc_dirty = cudaMemsetAsync(h->acc, 0, (size_t)B * h->N3 * sizeof(unsigned long long),
+                                   h->st) != cudaSuccess;
+  return r;
 }
 
 // Diagnostics record `idx` (the state after step idx - 1; idx 0 is the initial state).
@@ -1964,7 +1978,10 @@ static sim_status group_graph(sim_group_t* g, int kind, const std::vector<uintpt
                               Body body) {
   const size_t K = g->m.size();
   std::vector<HostState> before;
-  for (sim_t* h : g->m) before.push_back(snapshot(h));
+  for (sim_t* h : g->m) {
+    DH_TRY(settle_acc(h, g->st));
+    before.push_back(snapshot(h));
+  }
   for (GroupEntry& e : g->cache) {
     if (e.kind == kind && e.key == key && e.before == before) {
       DH_CUDA_TRY(cudaGraphLaunch(e.exec, g->st));
