@@ -29,6 +29,9 @@
  *     gives a message. Invalid arguments are rejected before any work is enqueued.
  *   - The library is not thread safe for one handle; distinct handles may be used from
  *     distinct threads.
+ *   - Entries without a handle take their scratch memory in the order of `stream`; at most
+ *     512 MB of it per device stays mapped between calls, until a handle is destroyed or an
+ *     allocation of the library fails.
  */
 #ifndef DIFFHYDRO_H
 #define DIFFHYDRO_H

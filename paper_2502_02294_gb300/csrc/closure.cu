@@ -720,7 +720,7 @@ static sim_status launch_conv(int mode, ConvArgs a, int B, cudaStream_t st) {
 // whatever N is. The epilogue adds the six blocks of each tap through shared memory and the
 // result to dW with vector atomics; the four epilogue warps of the dz = 0 CTAs also sum db
 // from the staged dz lines while the MMAs run.
-// Measured per layer: 33 us at 64^3 x 2 and 94 us at 128^3, against 303 us (64^3 x 2) for
+// Measured per layer: 33 us at 64^3 x 2 and 80 us at 128^3, against 303 us (64^3 x 2) for
 // im2col tiles transposed by stmatrix into K-major stages (N = 16), which spent its time on
 // 27 loads and stores per position.
 constexpr int DW_G = 6, DW_I = DW_G + 2;   // dz lines, input lines per stage
@@ -1188,6 +1188,11 @@ static void ws_free(sim_closure_s* c) {
 template <class T>
 static sim_status ws_alloc(sim_closure_s* c, T** p, size_t count) {
   cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    scratch_trim();
+    e = cudaMalloc((void**)p, count * sizeof(T));
+  }
   if (e != cudaSuccess) {
     set_error("closure: cudaMalloc(%zu bytes) failed: %s", count * sizeof(T), cudaGetErrorString(e));
     return SIM_ENOMEM;
@@ -1463,6 +1468,7 @@ void sim_closure_destroy(sim_closure_t* c) {
   for (void* p : {(void*)c->prm, (void*)c->grad, (void*)c->m, (void*)c->v, (void*)c->wf,
                   (void*)c->wb, (void*)c->err, (void*)c->loss})
     if (p) cudaFree(p);
+  scratch_trim();
   delete c;
 }
 
@@ -1599,7 +1605,7 @@ sim_status sim_refine_noise(const float* w_c, int32_t n_c, float* w_f, int32_t n
   const long long NCc = (long long)n_c * n_c * (n_c / 2 + 1);
   const long long NCf = (long long)n_f * n_f * (n_f / 2 + 1);
   cufftComplex* buf = nullptr;
-  DH_CUDA_TRY(cudaMallocAsync((void**)&buf, (NCc + NCf) * sizeof(cufftComplex), st));
+  DH_CUDA_TRY(scratch_alloc((void**)&buf, (NCc + NCf) * sizeof(cufftComplex), st));
   sim_status r = pc->set_stream(st);
   if (r == SIM_OK) r = pf->set_stream(st);
   if (r == SIM_OK && cufftExecR2C(pc->r2c1, const_cast<float*>(w_c), buf) != CUFFT_SUCCESS) {

@@ -14,6 +14,11 @@ namespace dh {
 // The last error message of the calling host thread (calls without a handle) is kept in a
 // thread-local buffer; handle calls also copy it into the handle.
 void set_error(const char* fmt, ...);
+
+// Stream-ordered scratch memory (free it with cudaFreeAsync) from a pool that keeps a bounded
+// amount mapped between calls; scratch_trim gives the current device's unused part back.
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st);
+void scratch_trim();
 const char* get_error();
 
 #define DH_CUDA_TRY(expr)                                                              \

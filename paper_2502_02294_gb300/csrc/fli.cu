@@ -229,12 +229,8 @@ extern "C" sim_status sim_cross_correlation(const float* a, const float* b, int3
   const long long NC = (long long)n * n * (n / 2 + 1);
   cufftComplex* buf = nullptr;
   double* sums = nullptr;
-  DH_CUDA_TRY(cudaMallocAsync((void**)&buf, 2 * NC * sizeof(cufftComplex), st));
-  if (cudaMallocAsync((void**)&sums, 5 * nbins * sizeof(double), st) != cudaSuccess) {
-    cudaFreeAsync(buf, st);
-    set_error("cudaMallocAsync failed");
-    return SIM_ENOMEM;
-  }
+  DH_CUDA_TRY(scratch_alloc((void**)&buf, 2 * NC * sizeof(cufftComplex) + 5 * nbins * sizeof(double), st));
+  sums = reinterpret_cast<double*>(buf + 2 * NC);
   sim_status r = plans->set_stream(st);
   if (r == SIM_OK && cudaMemsetAsync(sums, 0, 5 * nbins * sizeof(double), st) != cudaSuccess) {
     set_error("cudaMemsetAsync failed");
@@ -255,6 +251,5 @@ extern "C" sim_status sim_cross_correlation(const float* a, const float* b, int3
     }
   }
   cudaFreeAsync(buf, st);
-  cudaFreeAsync(sums, st);
   return r;
 }

@@ -1530,7 +1530,7 @@ extern "C" sim_status sim_sweep_adjoint(const float* u_in, const float* lam_out,
   // only the x march needs scratch (its transposed copies): 20 n^3 floats
   const bool need = axis == 0 && variant != SIM_SWEEP_TILE;
   float* scratch = nullptr;
-  if (need) DH_CUDA_TRY(cudaMallocAsync((void**)&scratch, 20ull * n * n * n * sizeof(float), st));
+  if (need) DH_CUDA_TRY(dh::scratch_alloc((void**)&scratch, 20ull * n * n * n * sizeof(float), st));
   const sim_status r =
       dh::launch_sweep_adjoint(axis, u_in, lam_out, lam_in, n, dh::sarg((float)nu), gamma,
                                limiter_eps, dh::dpart(dnu), scratch, 1, variant, st);

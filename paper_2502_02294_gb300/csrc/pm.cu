@@ -30,6 +30,7 @@ static sim_status make_plan(cufftHandle* h, int n, cufftType type, int batch) {
 }
 
 sim_status FFTPlans::create(int n_, int B_) {
+  scratch_trim();  // the plans take workspaces of their own
   n = n_;
   B = B_;
   DH_TRY(make_plan(&r2c1, n, CUFFT_R2C, B));
@@ -983,7 +984,7 @@ extern "C" sim_status sim_deposit_cic(const float* s, const float* values, int32
   cudaStream_t st = (cudaStream_t)stream;
   const long long N3 = (long long)n * n * n;
   unsigned long long* acc = nullptr;
-  DH_CUDA_TRY(cudaMallocAsync((void**)&acc, N3 * sizeof(unsigned long long), st));
+  DH_CUDA_TRY(scratch_alloc((void**)&acc, N3 * sizeof(unsigned long long), st));
   sim_status r = SIM_OK;
   if (cudaMemsetAsync(acc, 0, N3 * sizeof(unsigned long long), st) != cudaSuccess) {
     set_error("cudaMemsetAsync failed");
@@ -1015,7 +1016,7 @@ extern "C" sim_status sim_gravity(const float* delta, int32_t n, double box, dou
   cudaStream_t st = (cudaStream_t)stream;
   const long long NC = (long long)n * n * (n / 2 + 1);
   cufftComplex* buf = nullptr;
-  DH_CUDA_TRY(cudaMallocAsync((void**)&buf, 4 * NC * sizeof(cufftComplex), st));
+  DH_CUDA_TRY(scratch_alloc((void**)&buf, 4 * NC * sizeof(cufftComplex), st));
   sim_status r = launch_gravity(delta, g, buf, buf + NC, n, box,
                                 sarg(gravity_pref_norm(pref, n)), 1, *plans, st);
   cudaFreeAsync(buf, st);
@@ -1033,7 +1034,7 @@ extern "C" sim_status sim_gravity_adjoint(const float* lam_g, int32_t n, double 
   cudaStream_t st = (cudaStream_t)stream;
   const long long NC = (long long)n * n * (n / 2 + 1);
   cufftComplex* buf = nullptr;
-  DH_CUDA_TRY(cudaMallocAsync((void**)&buf, 4 * NC * sizeof(cufftComplex), st));
+  DH_CUDA_TRY(scratch_alloc((void**)&buf, 4 * NC * sizeof(cufftComplex), st));
   sim_status r = launch_gravity_adjoint(lam_g, lam_delta, buf, buf + 3 * NC, n, box,
                                         sarg(gravity_pref_norm(pref, n)), 1, *plans, st);
   cudaFreeAsync(buf, st);

@@ -211,6 +211,11 @@ static sim_status fail(sim_t* h, sim_status s) {
 
 static sim_status dalloc(sim_t* h, void** ptr, size_t bytes) {
   cudaError_t e = cudaMalloc(ptr, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    scratch_trim();
+    e = cudaMalloc(ptr, bytes);
+  }
   if (e != cudaSuccess) {
     set_error("cudaMalloc(%zu bytes) failed: %s", bytes, cudaGetErrorString(e));
     return SIM_ENOMEM;
@@ -1409,6 +1414,7 @@ void sim_destroy(sim_t* h) {
   h->plans1.destroy();
   for (void* a : h->allocs)
     if (a) cudaFree(a);
+  scratch_trim();
   delete h;
 }
 

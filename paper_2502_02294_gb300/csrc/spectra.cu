@@ -215,12 +215,8 @@ extern "C" sim_status sim_power_spectrum_adjoint(const float* a, int32_t n, doub
   const long long NC = (long long)n * n * (n / 2 + 1);
   cufftComplex* ak = nullptr;
   double* sums = nullptr;
-  DH_CUDA_TRY(cudaMallocAsync((void**)&ak, NC * sizeof(cufftComplex), st));
-  if (cudaMallocAsync((void**)&sums, nbins * sizeof(double), st) != cudaSuccess) {
-    cudaFreeAsync(ak, st);
-    set_error("cudaMallocAsync failed");
-    return SIM_ENOMEM;
-  }
+  DH_CUDA_TRY(scratch_alloc((void**)&ak, NC * sizeof(cufftComplex) + nbins * sizeof(double), st));
+  sums = reinterpret_cast<double*>(ak + NC);
   sim_status r = plans->set_stream(st);
   if (r == SIM_OK && cudaMemsetAsync(sums, 0, nbins * sizeof(double), st) != cudaSuccess) {
     set_error("cudaMemsetAsync failed");
@@ -248,7 +244,6 @@ extern "C" sim_status sim_power_spectrum_adjoint(const float* a, int32_t n, doub
     r = SIM_ECUDA;
   }
   cudaFreeAsync(ak, st);
-  cudaFreeAsync(sums, st);
   return r;
 }
 
@@ -265,13 +260,9 @@ extern "C" sim_status sim_power_spectrum(const float* a, const float* b, int32_t
   const long long NC = (long long)n * n * (n / 2 + 1);
   cufftComplex* buf = nullptr;
   double* sums = nullptr;
-  DH_CUDA_TRY(cudaMallocAsync((void**)&buf, 2 * NC * sizeof(cufftComplex), st));
+  DH_CUDA_TRY(scratch_alloc((void**)&buf, 2 * NC * sizeof(cufftComplex) + 3 * nbins * sizeof(double), st));
+  sums = reinterpret_cast<double*>(buf + 2 * NC);
   sim_status r = SIM_OK;
-  if (cudaMallocAsync((void**)&sums, 3 * nbins * sizeof(double), st) != cudaSuccess) {
-    cudaFreeAsync(buf, st);
-    set_error("cudaMallocAsync failed");
-    return SIM_ENOMEM;
-  }
   cufftComplex* ak = buf;
   cufftComplex* bk = b ? buf + NC : buf;
   if (plans->set_stream(st) != SIM_OK) r = SIM_ECUDA;
@@ -299,6 +290,5 @@ extern "C" sim_status sim_power_spectrum(const float* a, const float* b, int32_t
     }
   }
   cudaFreeAsync(buf, st);
-  cudaFreeAsync(sums, st);
   return r;
 }
