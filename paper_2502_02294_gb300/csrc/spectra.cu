@@ -19,7 +19,8 @@ __device__ __forceinline__ int mode_bin(int k2, float& root) {
   return b;
 }
 
-// (hi, lo) += v, v >= any size: error-free sum of float pairs
+// (hi, lo) += (v, vlo): float pairs, the sum hi + v by Knuth's two-sum (error-free while nothing
+// overflows; neither operand needs to be the larger)
 __device__ __forceinline__ void pair_add(float v, float vlo, float& hi, float& lo) {
   const float s = __fadd_rn(hi, v), t = __fsub_rn(s, hi);
   lo = __fadd_rn(lo, __fadd_rn(vlo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(v, t))));
@@ -36,10 +37,52 @@ __device__ __forceinline__ void run_sum(int lane, int last, float& hi, float& lo
   }
 }
 
-// hi + lo += x y, the product exact (hi, lo: unevaluated float pair, error-free sums)
-__device__ __forceinline__ void dot2(float x, float y, float& hi, float& lo) {
+__device__ __forceinline__ void run_sum(int lane, int last, double& v) {
+#pragma unroll 1
+  for (int d = 1; d < 32; d <<= 1) {
+    const double o = __shfl_down_sync(0xffffffffu, v, d);
+    if (lane + d <= last) v += o;
+  }
+}
+
+// hi + lo += x y as a float pair, the product exact while its low word stays representable
+// (kPairMin); m: the largest |product| so far
+__device__ __forceinline__ void dot2(float x, float y, float& hi, float& lo, float& m) {
   const float p = __fmul_rn(x, y);
   pair_add(p, __fmaf_rn(x, y, -p), hi, lo);
+  m = fmaxf(m, fabsf(p));
+}
+
+// Products for which float pairs are as good as doubles: a low word is a multiple of 2^-149,
+// 2^-59 of kPairMin, and the at most 512 products of a run stay below 2^110.
+constexpr float kPairMin = 0x1p-90f, kPairMax = 0x1p100f;
+
+// The powers of a warp's modes in FP64 (see spectrum_bin_kernel), added to the histogram once per
+// run of lanes; out of line, so that it costs the common path no registers.
+template <int NP>
+__device__ __noinline__ void spectrum_wide_run(const cufftComplex* a, const cufftComplex* b, int n,
+                                               int nbins, int kx, int ky, int kz, int bin,
+                                               bool two_y, bool two_z, int wx, int lane, int last,
+                                               bool head, double* hist) {
+  const unsigned nh = n / 2 + 1;
+#pragma unroll 1
+  for (int q = 0; q < NP; ++q) {  // |a|^2, |b|^2, Re(a conj b); NP = 1: the last alone
+    const cufftComplex* p = NP == 3 && q == 1 ? b : a;
+    const cufftComplex* r = NP == 3 && q == 0 ? a : b;
+    double v = 0.0;
+    if (bin >= 0)
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {
+        if (((c & 1) && !two_y) || ((c & 2) && !two_z)) continue;
+        const long long o =
+            ((long long)((c & 2) ? n - kz : kz) * n + ((c & 1) ? n - ky : ky)) * nh + kx;
+        const cufftComplex x = p[o], y = r[o];
+        v += (double)x.x * y.x + (double)x.y * y.y;
+      }
+    v *= (double)wx;
+    run_sum(lane, last, v);
+    if (head && bin >= 0) atomicAdd(hist + (size_t)(1 + q) * nbins + bin, v);
+  }
 }
 
 // Sums per bin 1 .. nbins: mode weight, weight |k|, and NP weighted powers (NP = 0: the weight
@@ -52,6 +95,10 @@ __device__ __forceinline__ void dot2(float x, float y, float& hi, float& lo) {
 // grows along a row; a shared-memory double atomic is a compare-and-swap loop). At 128^3, 64
 // bins, this took 80 us (108 us for NP = 3) with one FP64 update of every sum per mode, 21 us
 // (32 us) with one per thread; now 10 us (16 us).
+// A float pair has float's exponent range, the modes of a field in any units do not keep to it:
+// a warp with a product outside [kPairMin, kPairMax] (infinities among them) forms its powers
+// in FP64. For the cross product of NP = 3 the two auto products decide: its error counts
+// against the root of theirs.
 template <int NP>
 __global__ void __launch_bounds__(512) spectrum_bin_kernel(const cufftComplex* __restrict__ a,
                                                            const cufftComplex* __restrict__ b, int n,
@@ -85,9 +132,10 @@ __global__ void __launch_bounds__(512) spectrum_bin_kernel(const cufftComplex* _
     if (NP) {
       // |k| = root + (k2 - root^2) / (2 root) to 1e-14; mult is a power of two
       float khi = 0.0f, klo = 0.0f;
-      float hi[NP ? NP : 1], lo[NP ? NP : 1];
+      float hi[NP ? NP : 1], lo[NP ? NP : 1], m[NP ? NP : 1];
 #pragma unroll
-      for (int q = 0; q < NP; ++q) hi[q] = lo[q] = 0.0f;
+      for (int q = 0; q < NP; ++q) hi[q] = lo[q] = m[q] = 0.0f;
+      unsigned nzx = 0u, nzy = 0u;  // bits of the components: zero modes are exact
       if (bin >= 0) {
         const float fm = (float)mult;
         khi = fm * root;
@@ -99,13 +147,15 @@ __global__ void __launch_bounds__(512) spectrum_bin_kernel(const cufftComplex* _
               ((long long)((c & 2) ? n - kz : kz) * n + ((c & 1) ? n - ky : ky)) * nh + kx;
           const cufftComplex x = a[o], y = b[o];
           if (NP == 3) {
-            dot2(x.x, x.x, hi[0], lo[0]);
-            dot2(x.y, x.y, hi[0], lo[0]);
-            dot2(y.x, y.x, hi[1], lo[1]);
-            dot2(y.y, y.y, hi[1], lo[1]);
+            dot2(x.x, x.x, hi[0], lo[0], m[0]);
+            dot2(x.y, x.y, hi[0], lo[0], m[0]);
+            dot2(y.x, y.x, hi[1], lo[1], m[1]);
+            dot2(y.y, y.y, hi[1], lo[1], m[1]);
           }
-          dot2(x.x, y.x, hi[NP - 1], lo[NP - 1]);
-          dot2(x.y, y.y, hi[NP - 1], lo[NP - 1]);
+          dot2(x.x, y.x, hi[NP - 1], lo[NP - 1], m[NP - 1]);
+          dot2(x.y, y.y, hi[NP - 1], lo[NP - 1], m[NP - 1]);
+          nzx |= __float_as_uint(x.x) | __float_as_uint(x.y);
+          nzy |= __float_as_uint(y.x) | __float_as_uint(y.y);
         }
         const float fw = (float)wx;
 #pragma unroll
@@ -121,13 +171,23 @@ __global__ void __launch_bounds__(512) spectrum_bin_kernel(const cufftComplex* _
       const unsigned after = lane == 31 ? 0u : heads >> (lane + 1);
       const int last = after ? lane + __ffs(after) - 1 : 31;
       run_sum(lane, last, khi, klo);
+      if (head && bin >= 0) atomicAdd(hist + bin, (double)khi + (double)klo);
+      const bool zx = (nzx << 1) == 0u, zy = (nzy << 1) == 0u;
+      bool wide;
+      if (NP == 3)
+        wide = !(zx || (m[0] >= kPairMin && m[0] <= kPairMax)) ||
+               !(zy || (m[1] >= kPairMin && m[1] <= kPairMax));
+      else
+        wide = !(zx || zy || (m[0] >= kPairMin && m[0] <= kPairMax));
+      if (__any_sync(0xffffffffu, wide)) {
+        spectrum_wide_run<NP>(a, b, n, nbins, kx, ky, kz, bin, two_y, two_z, wx, lane, last, head, hist);
+      } else {
 #pragma unroll
-      for (int q = 0; q < NP; ++q) run_sum(lane, last, hi[q], lo[q]);
-      if (head && bin >= 0) {
-        atomicAdd(hist + bin, (double)khi + (double)klo);
+        for (int q = 0; q < NP; ++q) run_sum(lane, last, hi[q], lo[q]);
+        if (head && bin >= 0)
 #pragma unroll
-        for (int q = 0; q < NP; ++q)
-          atomicAdd(hist + (size_t)(1 + q) * nbins + bin, (double)hi[q] + (double)lo[q]);
+          for (int q = 0; q < NP; ++q)
+            atomicAdd(hist + (size_t)(1 + q) * nbins + bin, (double)hi[q] + (double)lo[q]);
       }
     }
   }
