@@ -271,31 +271,11 @@ __device__ __forceinline__ void vanleer_grad(float a, float b, float eps, float&
   if (ab > 0.0f) {
     const float s = a + b;
     const float D = s + copysignf(eps, s);
-    const float iD = fast_rcp(D);
-    const float i2 = iD * iD;
-    da = 2.0f * b * (D - a) * i2;
-    db = 2.0f * a * (D - b) * i2;
+    // one factor 1/D at a time: 1/D^2 overflows for |D| < 5e-20, where a b > 0 still holds
+    const float h = fast_rcp(D), q = 2.0f * h;
+    da = (b * q) * ((D - a) * h);
+    db = (a * q) * ((D - b) * h);
   } else {
-    da = 0.0f;
-    db = 0.0f;
-  }
-}
-
-// Limiter value and both partials in one pass (the adjoint needs the face flux for d/dnu):
-// phi as vanleer() up to the rounding of the reciprocal, da = dphi/da, db = dphi/db.
-__device__ __forceinline__ void vanleer_vg(float a, float b, float eps, float& phi, float& da,
-                                           float& db) {
-  const float ab = a * b;
-  if (ab > 0.0f) {
-    const float s = a + b;
-    const float D = s + copysignf(eps, s);
-    const float q = 2.0f * fast_rcp(D);  // 2 / D
-    const float q2 = 0.5f * q * q;       // 2 / D^2
-    phi = ab * q;
-    da = b * (D - a) * q2;
-    db = a * (D - b) * q2;
-  } else {
-    phi = 0.0f;
     da = 0.0f;
     db = 0.0f;
   }

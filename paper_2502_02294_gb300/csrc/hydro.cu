@@ -503,18 +503,20 @@ sweep_march2_kernel(const float* __restrict__ uin, float* __restrict__ uout, int
   }
 }
 
-// Limiter value and both partials of two lanes, as vanleer_vg (branch-free: the gate selects
-// per lane after the arithmetic of both).
+// Limiter value and both partials of two lanes, as vanleer and vanleer_grad, in one pass (the
+// adjoint needs the face flux for d/dnu; branch-free: the gate selects per lane after the
+// arithmetic of both).
 __device__ __forceinline__ void vanleer_vg2(float2 a, float2 b, float eps, float2& phi, float2& da,
                                             float2& db) {
   const float2 ab = mul2(a, b);
   const float2 s = add2(a, b);
   const float2 D = add2(s, make_float2(copysignf(eps, s.x), copysignf(eps, s.y)));
-  const float2 q = mul2(pk(2.0f), make_float2(fast_rcp(D.x), fast_rcp(D.y)));  // 2 / D
-  const float2 q2 = mul2(mul2(q, q), pk(0.5f));                                  // 2 / D^2
+  const float2 h = make_float2(fast_rcp(D.x), fast_rcp(D.y));  // 1 / D
+  const float2 q = mul2(pk(2.0f), h);
   const float2 p = mul2(ab, q);
-  const float2 dA = mul2(mul2(b, sub2(D, a)), q2);
-  const float2 dB = mul2(mul2(a, sub2(D, b)), q2);
+  // one factor 1 / D at a time (see vanleer_grad)
+  const float2 dA = mul2(mul2(b, q), mul2(sub2(D, a), h));
+  const float2 dB = mul2(mul2(a, q), mul2(sub2(D, b), h));
   const bool gx = ab.x > 0.0f, gy = ab.y > 0.0f;
   phi = make_float2(gx ? p.x : 0.0f, gy ? p.y : 0.0f);
   da = make_float2(gx ? dA.x : 0.0f, gy ? dA.y : 0.0f);
