@@ -617,7 +617,13 @@ sweep_adj_march_kernel(const float* __restrict__ uin, const float* __restrict__ 
   const uint32_t bua = (uint32_t)__cvta_generic_to_shared(&bu[0][0][tid]);
   const uint32_t bla = (uint32_t)__cvta_generic_to_shared(&bl[0][0][tid]);
   constexpr uint32_t kField = 128 * sizeof(float);
-  const int ww = live ? w : 0;
+  // Lanes past the row's end go along (the block sums need them) on stand-in cells of the row, each
+  // on its own: with one cell for all of them, every copy of one global word to many shared ones
+  // took a shared-memory pass per lane (3.5 M passes in a 65^3 march of 4 M warp instructions).
+  // y at 33^3 / 48^3 / 65^3 / 97^3 / 144^3 19.4 / 18.5 / 50 / 63 / 108 -> 10.1 / 14.5 / 23 / 45 / 96
+  // us, full rows as before. (Dead lanes that copy nothing cost a predicate per copy: 128^3 69.4 ->
+  // 70.9 us.)
+  const int ww = w < n ? w : (w - n) % n;
   const long long step = AXIS == 0 ? 1 : (AXIS == 1 ? n : (long long)n * n);
   auto fetch = [&](long long o, int it) {
 #pragma unroll
