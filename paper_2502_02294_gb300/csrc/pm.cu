@@ -126,28 +126,26 @@ struct PIdx {
   bool ok;
 };
 
-// Lattice site of a thread. BT > 0: a block of BT threads covers a brick of lattice sites, 32
-// (n a multiple of 32) or 16 sites in x, 4 in z for BT = 512 and 2 below, the rest in y; grid
-// (bricks in x times y, bricks in z, B). The CIC corners of a brick lie on few node rows, so
-// its warps share them in L1. BT = 0: blocks of 128 consecutive sites, grid (cdiv(n^3, 128),
-// B). Lanes without a particle get ok = false (and a lattice site past the end, never used).
-// In both, neighbouring lanes hold neighbouring x sites.
-__host__ __device__ constexpr int brick_lz(int bt) { return bt >= 512 ? 2 : 1; }
-__host__ __device__ constexpr int brick_lt(int bt) { return bt >= 512 ? 9 : (bt >= 256 ? 8 : 7); }
+// Lattice site of a thread. BRICK: a block of 256 threads covers a brick of lattice sites, 32 x 4
+// x 2 (n a multiple of 32) or 16 x 8 x 2, grid (bricks in x times y, bricks in z, B). The CIC
+// corners of a brick lie on few node rows, so its warps share them in L1. Otherwise: blocks of
+// 128 consecutive sites, grid (cdiv(n^3, 128), B). Lanes without a particle get ok = false (and a
+// lattice site past the end, never used). In both, neighbouring lanes hold neighbouring x sites.
+constexpr int kBrick = 256;  // threads (and sites) of a brick
+__host__ __device__ __forceinline__ int brick_lx(int n) { return (n & 31) == 0 ? 5 : 4; }
 
-template <int BT>
+template <bool BRICK>
 __device__ __forceinline__ PIdx particle_index(int n) {
   PIdx r;
-  if (BT > 0) {
-    constexpr int lz = brick_lz(BT), lt = brick_lt(BT);
-    const int lx = (n & 31) == 0 ? 5 : 4, ly = lt - lz - lx;
+  if (BRICK) {
+    const int lx = brick_lx(n), ly = 7 - lx;
     const int nbx = (n + (1 << lx) - 1) >> lx;
     const int by = blockIdx.x / nbx, bx = blockIdx.x - by * nbx;
     const int t = threadIdx.x;
     r.b = blockIdx.z;
     r.qx = (bx << lx) + (t & ((1 << lx) - 1));
     r.qy = (by << ly) + ((t >> lx) & ((1 << ly) - 1));
-    r.qz = (blockIdx.y << lz) + (t >> (lt - lz));
+    r.qz = 2 * blockIdx.y + (t >> 7);
     r.ok = r.qx < n && r.qy < n && r.qz < n;
     r.p = (r.qz * n + r.qy) * n + r.qx;
     return r;
@@ -175,31 +173,42 @@ __device__ __forceinline__ PIdx particle_index(int n) {
 
 constexpr int kPT = 128;  // threads per block of consecutive sites
 
-// Threads per brick of the particle kernels that gain from them. Late in a 128^3 run (flow of
-// several cells) the kick adjoint takes 106 us with bricks of 256 (108 with 512, 132 with 128)
-// against 129 us with consecutive sites, the readout of three fields 40 us against 50. The
-// kick (54 us against 57-58), the deposit (29 against 31) and its adjoint (47, the same) keep
-// consecutive sites: their blocks reuse little across rows, and the finer order balances
-// better.
-constexpr int kBrickKickAdj = 256, kBrickInterp = 256;
-
-// Bricks where they give every SM two blocks or more; small grids keep the finer blocks.
-static inline bool use_bricks(int bt, int n, int B) {
-  return (long long)n * n * n * B >= 2ll * 152 * bt;
-}
-static inline dim3 particle_grid(int bt, int n, int B) {
-  if (bt == 0) return dim3((unsigned)cdiv((long long)n * n * n, kPT), B);
-  const int lx = n % 32 == 0 ? 5 : 4, lz = brick_lz(bt), ly = brick_lt(bt) - lz - lx;
-  return dim3(cdiv(n, 1 << lx) * cdiv(n, 1 << ly), cdiv(n, 1 << lz), B);
+static inline dim3 particle_grid(bool brick, int n, int B) {
+  if (!brick) return dim3((unsigned)cdiv((long long)n * n * n, kPT), B);
+  const int lx = brick_lx(n);
+  return dim3(cdiv(n, 1 << lx) * cdiv(n, 1 << (7 - lx)), cdiv(n, 2), B);
 }
 
-// launch of a particle kernel with bricks of BT threads or consecutive sites
-#define DH_LAUNCH_PARTICLES(kernel, BT, n, B, st, ...)                                          \
+// Bricks for the kernels that gain from them, the kick adjoint and the readout. Late in a 128^3 run
+// (flow of several cells) the kick adjoint takes 105 us with bricks (108 with 512 sites, 132 with
+// 128) against 126 with consecutive sites, the readout of three fields 40 against 51. The kick
+// (54 us against 57-58), the deposit (29 against 31) and its adjoint (47, the same) keep
+// consecutive sites: their blocks reuse little across rows, and the finer order balances better.
+// A brick that overhangs the lattice has idle lanes, up to half as many as particles where n is
+// just above a multiple of 16, so bricks are taken where
+//   - they give every SM two blocks or more (small grids keep the finer blocks), and
+//   - the idle lanes are at most idle16 sixteenths of the particles.
+// Consecutive -> bricks, us, by n (idle lanes per particle). Readout, which takes up to 1/4:
+// 49 (.52) 6.0 -> 7.1, 50 (.43) 6.3 -> 7.1, 65 (.38) 10.1 -> 10.6, 97 (.25) 23.9 -> 23.2, 145 (.17) 77
+// -> 66, 80 (0) 14.7 -> 12.9. Kick adjoint, which gains more the larger the grid: 48 (0) 8.7 -> 8.4,
+// 72 (.11) 24.2 -> 24.6, 96 (0) 49.2 -> 48.1, 100 (.17) 57 -> 62, 112 (0) 82 -> 75, 129 (.19) 129 -> 127,
+// 161 (.15) 266 -> 238, 225 (.11) 757 -> 630, but 49 (.52) 9.3 -> 13.5, 65 (.38) 18.0 -> 23.2, 97 (.25)
+// 51 -> 60.
+static bool use_bricks(int n, int B, int idle16) {
+  const long long n3 = (long long)n * n * n;
+  const dim3 g = particle_grid(true, n, 1);
+  return n3 * B >= 2ll * 152 * kBrick && ((long long)g.x * g.y * kBrick - n3) * 16 <= idle16 * n3;
+}
+constexpr int kInterpIdle16 = 4;
+static int kick_adj_idle16(int n) { return n >= 112 ? 3 : (n >= 96 ? 1 : 0); }
+
+// launch of a particle kernel with bricks or consecutive sites
+#define DH_LAUNCH_PARTICLES(kernel, idle16, n, B, st, ...)                                      \
   do {                                                                                          \
-    if (use_bricks(BT, n, B))                                                                   \
-      DH_CUDA_TRY((launch_pdl(kernel<BT>, particle_grid(BT, n, B), BT, 0, st, __VA_ARGS__)));   \
+    if (use_bricks(n, B, idle16))                                                               \
+      DH_CUDA_TRY((launch_pdl(kernel<true>, particle_grid(true, n, B), kBrick, 0, st, __VA_ARGS__))); \
     else                                                                                        \
-      DH_CUDA_TRY((launch_pdl(kernel<0>, particle_grid(0, n, B), kPT, 0, st, __VA_ARGS__)));    \
+      DH_CUDA_TRY((launch_pdl(kernel<false>, particle_grid(false, n, B), kPT, 0, st, __VA_ARGS__))); \
     DH_LAUNCH_CHECK();                                                                          \
   } while (0)
 
@@ -265,7 +274,7 @@ __global__ void __launch_bounds__(128, 16) deposit_kernel(const float* __restric
                                                           unsigned long long* __restrict__ acc) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index<0>(n);  // lanes past the last particle stay for the warp exchange
+  const PIdx q = particle_index<false>(n);  // lanes past the last particle stay for the warp exchange
   s += (size_t)q.b * 3 * N3;
   acc += (size_t)q.b * N3;
   Cic c;
@@ -343,7 +352,7 @@ __global__ void fix_to_float_kernel(const unsigned long long* __restrict__ acc, 
 
 sim_status launch_deposit(const float* s, const float* values, int n, float inv_dx,
                           unsigned long long* acc, int B, cudaStream_t st) {
-  const dim3 grid = particle_grid(0, n, B);
+  const dim3 grid = particle_grid(false, n, B);
   if (values)
     DH_CUDA_TRY((launch_pdl(deposit_kernel<false>, grid, kPT, 0, st, s, values, n, inv_dx, acc)));
   else
@@ -495,12 +504,12 @@ sim_status launch_gravity_adjoint(const float* lam_g, float* lam_delta, cufftCom
 }
 
 // ------------------------------------------------------------------ readout, kick, drift
-template <int BT>
+template <bool BRICK>
 __global__ void interp_kernel(const float* __restrict__ grid, int nf, int n, float inv_dx,
                               const float* __restrict__ s, float* __restrict__ out) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index<BT>(n);
+  const PIdx q = particle_index<BRICK>(n);
   if (!q.ok) return;
   grid += (size_t)q.b * nf * N3;
   s += (size_t)q.b * 3 * N3;
@@ -523,7 +532,7 @@ __global__ void interp_kernel(const float* __restrict__ grid, int nf, int n, flo
 
 sim_status launch_interp(const float* grid, int nf, int n, float inv_dx, const float* s,
                          float* out, int B, cudaStream_t st) {
-  DH_LAUNCH_PARTICLES(interp_kernel, kBrickInterp, n, B, st, grid, nf, n, inv_dx, s, out);
+  DH_LAUNCH_PARTICLES(interp_kernel, kInterpIdle16, n, B, st, grid, nf, n, inv_dx, s, out);
   return SIM_OK;
 }
 
@@ -556,7 +565,7 @@ __global__ void __launch_bounds__(128, 16) kick_drift_kernel(const float* s, flo
                                   int n, float inv_dx) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index<0>(n);
+  const PIdx q = particle_index<false>(n);
   if (!q.ok) return;
   const int i = q.p;
   const size_t o3 = (size_t)q.b * 3 * N3;
@@ -595,7 +604,7 @@ __global__ void __launch_bounds__(128, 16) kick_drift_kernel(const float* s, flo
 sim_status launch_kick_drift(const float* s, float* s_out, const float* p, float* p_out,
                              const float* g, SArg K, SArg dtau, const float* zhat, float* aux,
                              int n, float inv_dx, int B, cudaStream_t st) {
-  DH_CUDA_TRY((launch_pdl(kick_drift_kernel, particle_grid(0, n, B), kPT, 0, st, s, s_out, p,
+  DH_CUDA_TRY((launch_pdl(kick_drift_kernel, particle_grid(false, n, B), kPT, 0, st, s, s_out, p,
                           p_out, g, K, dtau, zhat, aux, n, inv_dx)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
@@ -634,7 +643,7 @@ sim_status launch_gas_kick(const float* in, float* out, const float* g, SArg K, 
 // Adjoint of kick_drift_kernel: the particle part and, when lam_gas is not NULL, the gas
 // kick of the cell with the same index at the pre-kick gas state gas_u (its force adjoint
 // goes to lam_g4 with a float4 atomic: other particles scatter into the node concurrently).
-template <int BT>
+template <bool BRICK>
 __global__ void kick_drift_adj_kernel(const float* __restrict__ s0, const float* __restrict__ p0,
                                       const float* __restrict__ g, SArg Ka, SArg dtaua,
                                       float* __restrict__ lam_s, float* __restrict__ lam_p,
@@ -643,7 +652,7 @@ __global__ void kick_drift_adj_kernel(const float* __restrict__ s0, const float*
                                       int n, float inv_dx) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index<BT>(n);
+  const PIdx q = particle_index<BRICK>(n);
   const size_t o3 = (size_t)q.b * 3 * N3;
   s0 += o3;
   if (p0) p0 += o3;
@@ -766,7 +775,7 @@ sim_status launch_kick_drift_adjoint(const float* s0, const float* p0, const flo
                                      SArg dtau, float* lam_s, float* lam_p, float4* lam_g4,
                                      DPart dK, DPart ddtau, const float* gas_u, float* lam_gas,
                                      int n, float inv_dx, int B, cudaStream_t st) {
-  DH_LAUNCH_PARTICLES(kick_drift_adj_kernel, kBrickKickAdj, n, B, st, s0, p0, g, K, dtau, lam_s, lam_p, lam_g4, dK,
+  DH_LAUNCH_PARTICLES(kick_drift_adj_kernel, kick_adj_idle16(n), n, B, st, s0, p0, g, K, dtau, lam_s, lam_p, lam_g4, dK,
                       ddtau, gas_u, lam_gas, n, inv_dx);
   return SIM_OK;
 }
@@ -778,7 +787,7 @@ __global__ void __launch_bounds__(128, 16) deposit_adj_kernel(const float* __res
                                    long long rho_stride) {
   pdl_enter();
   const int N3 = n * n * n;
-  const PIdx q = particle_index<0>(n);
+  const PIdx q = particle_index<false>(n);
   s += (size_t)q.b * 3 * N3;
   lam_s += (size_t)q.b * 3 * N3;
   ld += (size_t)q.b * N3;
@@ -812,7 +821,7 @@ __global__ void __launch_bounds__(128, 16) deposit_adj_kernel(const float* __res
 sim_status launch_deposit_adjoint(const float* s, const float* lam_delta, SArg cm,
                                   float* lam_s, DPart dcm, int n, float inv_dx, int B,
                                   cudaStream_t st, float* lam_rho, long long rho_stride) {
-  DH_CUDA_TRY((launch_pdl(deposit_adj_kernel, particle_grid(0, n, B), kPT, 0, st, s, lam_delta,
+  DH_CUDA_TRY((launch_pdl(deposit_adj_kernel, particle_grid(false, n, B), kPT, 0, st, s, lam_delta,
                           cm, lam_s, dcm, n, inv_dx, lam_rho, rho_stride)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
