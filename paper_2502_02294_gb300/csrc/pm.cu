@@ -780,8 +780,12 @@ sim_status launch_kick_drift_adjoint(const float* s0, const float* p0, const flo
   return SIM_OK;
 }
 
-// 32 registers instead of 40 (2,048 resident threads per SM): 48.6 -> 42.2 us at 128^3
-__global__ void __launch_bounds__(128, 16) deposit_adj_kernel(const float* __restrict__ s, const float* __restrict__ ld,
+// MB resident blocks per SM: 16 hold the registers at 32 instead of 40 (2,048 resident threads),
+// 48.5 -> 42.0 us at 128^3. A grid that 13 blocks per SM cover (n <= 63) gains nothing from more and
+// keeps the registers for loads in flight: 32^3 / 48^3 / 60^3 3.97 / 5.26 / 7.15 us with 16, 3.36 /
+// 4.64 / 6.70 with 12 (64^3 7.4 against 7.5).
+template <int MB>
+__global__ void __launch_bounds__(128, MB) deposit_adj_kernel(const float* __restrict__ s, const float* __restrict__ ld,
                                    SArg cma, float* __restrict__ lam_s, DPart dcm, int n,
                                    float inv_dx, float* __restrict__ lam_rho,
                                    long long rho_stride) {
@@ -821,8 +825,10 @@ __global__ void __launch_bounds__(128, 16) deposit_adj_kernel(const float* __res
 sim_status launch_deposit_adjoint(const float* s, const float* lam_delta, SArg cm,
                                   float* lam_s, DPart dcm, int n, float inv_dx, int B,
                                   cudaStream_t st, float* lam_rho, long long rho_stride) {
-  DH_CUDA_TRY((launch_pdl(deposit_adj_kernel, particle_grid(false, n, B), kPT, 0, st, s, lam_delta,
-                          cm, lam_s, dcm, n, inv_dx, lam_rho, rho_stride)));
+  const dim3 grid = particle_grid(false, n, B);
+  auto kernel = (long long)grid.x * B <= 13ll * 152 ? deposit_adj_kernel<12> : deposit_adj_kernel<16>;
+  DH_CUDA_TRY((launch_pdl(kernel, grid, kPT, 0, st, s, lam_delta, cm, lam_s, dcm, n, inv_dx, lam_rho,
+                          rho_stride)));
   DH_LAUNCH_CHECK();
   return SIM_OK;
 }
