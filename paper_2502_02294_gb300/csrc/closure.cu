@@ -714,18 +714,29 @@ static sim_status launch_conv(int mode, ConvArgs a, int B, cudaStream_t st) {
 // (M = 2 x 8 x 8 = 128 rows), for a run of xs positions. One MMA over 16 positions correlates
 // every input line with every dz line: the blocks (i, j) with i - j - 1 = dy in {-1, 0, 1}
 // are the three dy taps (18 of the 48 blocks, the others are not read), dx is a shift of the
-// A operand by one position. The accumulators of the three dx take 3 x 96 of the 512 TMEM
-// columns and collect all of the CTA's stages; dz is the CTA's blockIdx.y, which triples the
-// reads (from L2) but lets N be 96: an MMA reads its 4 KB A operand from shared memory
-// whatever N is. The epilogue adds the six blocks of each tap through shared memory and the
-// result to dW with vector atomics; the four epilogue warps of the dz = 0 CTAs also sum db
-// from the staged dz lines while the MMAs run.
-// Measured per layer: 33 us at 64^3 x 2 and 80 us at 128^3, against 303 us (64^3 x 2) for
-// im2col tiles transposed by stmatrix into K-major stages (N = 16), which spent its time on
-// 27 loads and stores per position.
+// A operand by one position. dz is the CTA's blockIdx.y, which triples the reads (from L2) but
+// lets N be 96: an MMA reads its 4 KB A operand from shared memory whatever N is.
+// An accumulator collects a chain of at most DW_CHAIN MMAs: the tensor core's float32 sums lose
+// bits in proportion to the chain (not to its root), so a chain over all of a CTA's stages, 456
+// MMAs at 128^3, was 1.6e-5 off for a sum of one sign, more than the im2col kernel's chains (5.4e-6).
+// Five accumulators of 96 columns take turns: the MMAs of dx = 0 and 1 of the next chain run into
+// the two spare ones while the epilogue warps add the chain before it to their registers (the 18
+// blocks, one row of one block per lane and dx, dy), and dx = 2 follows into the first one drained.
+// At the end the epilogue adds the six blocks of each tap through shared memory and the result to
+// dW with vector atomics. Two more warps sum db from the staged dz lines while the MMAs run, each of
+// the three dz CTAs (which stage the same lines) a third of the stages: all of it in one of them
+// made that one wait (shared-memory bandwidth; 102 us per 128^3 launch against 94).
+// Measured per layer, launches overlapped: 34 us at 64^3 x 2 and 73 us at 128^3 (33 and 80 with one
+// chain per CTA and db in the epilogue warps), against 303 us (64^3 x 2) for im2col tiles
+// transposed by stmatrix into K-major stages (N = 16), which spent its time on 27 loads and stores
+// per position. Relative error of the last layer's dW against 64 bits, gradients of one sign, 64^3
+// x 2 / 128^3 / 193^3: 4.3e-7 / 4.6e-7 / 3.5e-7 (one chain 2.1e-6 / 1.6e-5 / 8.7e-5, im2col 9e-7 /
+// 5.4e-6 / 3.5e-5).
 constexpr int DW_G = 6, DW_I = DW_G + 2;   // dz lines, input lines per stage
 constexpr int DW_NC = 16 * DW_G;           // accumulator columns of one dx
-constexpr int DW_THREADS = 192;            // loader warp, MMA warp, four epilogue warps
+constexpr int DW_SLOTS = 5;                // accumulators (5 x 96 of the 512 TMEM columns)
+constexpr int DW_CHAIN = 32;               // MMAs of one chain, at most
+constexpr int DW_THREADS = 256;            // loader warp, MMA warp, four epilogue warps, two for db
 constexpr int DW_MAX_STAGES = 6;
 constexpr int DW_XS = 128;                 // positions per stage, at most
 constexpr int DW_RED = DW_I * 3 * 256 * 4;  // bytes of the epilogue's partial sums
@@ -740,6 +751,7 @@ struct DwArgs {
   int g_whole;     // dz lines staged whole with their padding (n a multiple of 16, nseg = 1)
   int stages, stage_bytes;
   int units, per_cta;  // stages of one dz, stages of one CTA
+  int chain;           // stages of one chain of MMAs
   float* dW;  // [27][16][16], accumulated
   float* db;  // [16], accumulated
   int* err;
@@ -789,13 +801,13 @@ __device__ __forceinline__ void tmem_ld8x2(uint32_t t0, uint32_t t1, float v[16]
 __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ uint64_t full[DW_MAX_STAGES], empty[DW_MAX_STAGES], done;
+  __shared__ uint64_t chained, drained[DW_SLOTS];  // a chain's MMAs done; an accumulator read
   __shared__ uint32_t tslot;
   __shared__ int sflag;
-  __shared__ float bred[4][16];
+  __shared__ float bred[2][16];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int n = a.n, S = a.stages;
   const int dz = (int)blockIdx.y - 1;
-  const bool bias = dz == 0;  // this CTA also sums db
   const int u0 = blockIdx.x * a.per_cta;
   const int nu = min(a.per_cta, a.units - u0);  // >= 1 by the launch
   const uint32_t s0 = smem_u32(smem);
@@ -811,23 +823,27 @@ __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
   if (tid == 0) {
     for (int st = 0; st < S; ++st) {
       mbar_init(full + st, 1);
-      mbar_init(empty + st, bias ? 5 : 1);
+      mbar_init(empty + st, 3);
     }
     mbar_init(&done, 1);
+    mbar_init(&chained, 1);
+    for (int i = 0; i < DW_SLOTS; ++i) mbar_init(drained + i, 4);
     sflag = 0;
   }
   if (w == 0) tmem_alloc_warp(&tslot, 512u);
   fence_async_smem();
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = tslot;
-  if (w < 4) tmem_zero(tmem, 0, 3 * DW_NC, w, 1);
   pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  const uint32_t tmem = tslot;
+  const bool one_chain = nu <= a.chain;
 
+  float acc[3][3][16];  // epilogue warps: [dx][dy + 1] of this lane's (input line, channel)
+#pragma unroll
+  for (int d = 0; d < 9; ++d)
+#pragma unroll
+    for (int c = 0; c < 16; ++c) acc[d / 3][d % 3][c] = 0.0f;
   float bacc[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) bacc[c] = 0.0f;
@@ -901,99 +917,156 @@ __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
     const uint64_t a_base = umma_desc(s0, 128u, pi), b_base = umma_desc(s0 + g_off + g_x0, 128u, pg);
     const uint32_t a_hi = (uint32_t)(a_base >> 32), b_hi = (uint32_t)(b_base >> 32);
     int committed = 0, st = 0, par = 0, seg = u0 % a.nseg;
-    for (int k = 0; k < nu; ++k) {
-      const uint32_t ok = mbar_wait_ns(full + st, par, limit);
-      if (!__all_sync(0xffffffffu, ok)) {
-        sflag = 1;
-        break;
+    int left = 0;           // stages until the chain ends
+    uint32_t use = 0u - 3u;  // 3 x chain; chain c holds dx in accumulator (3 c + dx) mod 5
+    bool ok = true;
+    for (int k = 0; k < nu && ok; ++k) {
+      const bool first = left == 0;
+      if (first) {
+        left = a.chain;
+        use += 3;
       }
+      ok = __all_sync(0xffffffffu, mbar_wait_ns(full + st, par, limit));
+      if (!ok) break;
       tc_fence_after();
       const int steps = (min(a.xs, n - seg * a.xs) + 15) >> 4;
       // descriptors are linear in the start address (16-byte units: one per position)
       const uint32_t off = (uint32_t)(st * a.stage_bytes) >> 4;
       const uint32_t a_lo = (uint32_t)a_base + off, b_lo = (uint32_t)b_base + off;
 #pragma unroll
-      for (int dx = 0; dx < 3; ++dx)
+      for (int dx = 0; dx < 3; ++dx) {
+        const uint32_t slot = (use + dx) % DW_SLOTS, turn = (use + dx) / DW_SLOTS;
+        if (first && turn > 0) {  // the chain that held it before has been read
+          ok = __all_sync(0xffffffffu, mbar_wait_ns(drained + slot, (turn - 1) & 1, limit));
+          if (!ok) break;
+          tc_fence_after();
+        }
 #pragma unroll
         for (int q = 0; q < DW_XS / 16; ++q)
           if (q < steps)
-            umma_bf16_acc(leader, tmem + (uint32_t)(dx * DW_NC), a_lo + (uint32_t)(16 * q + dx), a_hi,
-                          b_lo + (uint32_t)(16 * q), b_hi, idesc);
-      umma_commit(leader, empty + st);
+            umma_bf16(leader, tmem + slot * DW_NC, a_lo + (uint32_t)(16 * q + dx), a_hi,
+                      b_lo + (uint32_t)(16 * q), b_hi, idesc, !first || q > 0);
+      }
       committed = k + 1;
+      if (!ok) break;
+      umma_commit(leader, empty + st);
+      if (--left == 0 || k + 1 == nu) umma_commit(leader, &chained);
       if (++seg == a.nseg) seg = 0;
       if (++st == S) {
         st = 0;
         par ^= 1;
       }
     }
+    if (!ok) sflag = 1;
     if (committed > 0) {
-      // completes once every MMA issued above has; waited for before TMEM is read or freed
+      // completes once every MMA issued above has; waited for before TMEM is freed
       umma_commit(leader, &done);
       if (!mbar_wait_ns(&done, 0, kDrainNs)) sflag = 1;
     }
     __syncwarp();
-  } else if (bias) {
-    // ---- db: thread t of the four warps sums half t & 1 of the positions t / 2 mod 64
-    const int t = tid - 64, h = t & 1;
+  } else if (w >= 6) {
+    // ---- db: thread t of the two warps sums half t & 1 of the positions t / 2 mod 32 of every
+    //      third stage
+    const int t = tid - 192, h = t & 1;
     DwUnit u(a, u0);
+    int st = 0, par = 0, third = 0;
     for (int k = 0; k < nu; ++k, u.next(a)) {
-      const int st = k % S;
-      uint32_t ok = 0;
-      if (lane == 0) ok = mbar_wait_ns(full + st, (k / S) & 1, limit);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) {
-        if (lane == 0) sflag = 1;
+      if (!__all_sync(0xffffffffu, mbar_wait_ns(full + st, par, limit))) {
+        sflag = 1;
         break;
       }
       const int xn = u.xn(a), nl = u.lines(a);
       const uint8_t* g = smem + (size_t)st * a.stage_bytes + g_off + g_x0 + (size_t)(DW_G * h) * pg;
-      for (int j = 0; j < nl; ++j)
-        for (int x = t >> 1; x < xn; x += 64) {
-          const uint4 v = *reinterpret_cast<const uint4*>(g + (size_t)j * pg + (size_t)x * 16);
-          const uint32_t q[4] = {v.x, v.y, v.z, v.w};
+      const int x0 = third == (int)blockIdx.y ? t >> 1 : xn;
+      for (int x = x0; x < xn; x += 32) {
+        uint4 v[DW_G];
+#pragma unroll
+        for (int j = 0; j < DW_G; ++j)
+          v[j] = j < nl ? *reinterpret_cast<const uint4*>(g + (size_t)j * pg + (size_t)x * 16)
+                        : make_uint4(0u, 0u, 0u, 0u);
+        float p[8];  // the six lines first: short chains
+#pragma unroll
+        for (int c = 0; c < 8; ++c) p[c] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < DW_G; ++j) {
+          const uint32_t q[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            bacc[2 * c] += __uint_as_float(q[c] << 16);  // a bfloat16 is the high half of a float
-            bacc[2 * c + 1] += __uint_as_float(q[c] & 0xffff0000u);
+            p[2 * c] += __uint_as_float(q[c] << 16);  // a bfloat16 is the high half of a float
+            p[2 * c + 1] += __uint_as_float(q[c] & 0xffff0000u);
           }
         }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) bacc[c] += p[c];
+      }
+      if (++third == 3) third = 0;
       __syncwarp();
-      if (lane == 0) {
-        uint64_t state;
-        asm volatile("mbarrier.arrive.shared::cta.b64 %0, [%1];"
-                     : "=l"(state)
-                     : "r"(smem_u32(empty + st))
-                     : "memory");
-        (void)state;
+      if (lane == 0) mbar_arrive(empty + st);
+      if (++st == S) {
+        st = 0;
+        par ^= 1;
       }
     }
+  } else {
+    // ---- epilogue: TMEM lane 8 (8 h + i) + c8 of warp w % 4 holds half h = (w % 4) / 2, input
+    //      lines i0 .. i0 + 3; columns 8 (6 h' + j) + c8'
+    const int i0 = 4 * (w & 1), il = lane >> 3;
+    const uint32_t tl = tmem + ((uint32_t)(32 * (w & 3)) << 16);
+    bool ok = true;
+    uint32_t use = 0, turn = 0;
+    // (a CTA with one chain leaves it in TMEM)
+    for (int k = one_chain ? nu : 0; k < nu && ok; k += a.chain, use += 3, ++turn) {
+      ok = __all_sync(0xffffffffu, mbar_wait_ns(&chained, turn & 1, limit));
+      if (!ok) break;
+      tc_fence_after();
+#pragma unroll
+      for (int dx = 0; dx < 3; ++dx) {
+        const uint32_t slot = (use + dx) % DW_SLOTS, ts = tl + slot * DW_NC;
+#pragma unroll
+        for (int jj = 0; jj < 6; ++jj) {
+          const int j = i0 - 2 + jj;  // the same for the whole warp
+          if (j < 0 || j >= DW_G) continue;
+          float v[16];
+          tmem_ld8x2(ts + (uint32_t)(8 * j), ts + (uint32_t)(8 * (DW_G + j)), v);
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            // dy + 1 = d is the input line j + d
+            if (il == jj + d - 2)
+#pragma unroll
+              for (int c = 0; c < 16; ++c) acc[dx][d][c] += v[c];
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(drained + slot);
+      }
+    }
+    if (!ok) sflag = 1;
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (w >= 2 && sflag == 0) {
-    // TMEM lane 8 (8 h + i) + c8 of warp w % 4: half h = q / 2, input lines i0 .. i0 + 3;
-    // columns 8 (6 h' + j) + c8'
-    const int t = tid - 64, q = w & 3;
-    const int i0 = 4 * (q & 1), i = i0 + (lane >> 3), ci = 8 * (q >> 1) + (lane & 7);
-    const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
-    float* red = reinterpret_cast<float*>(smem);  // [i][dy + 1][ci][co]
-#pragma unroll 1
-    for (int dx = 0; dx < 3; ++dx) {
-#pragma unroll 1
-      for (int j = max(0, i0 - 2); j < min(DW_G, i0 + 4); ++j) {  // the same for the whole warp
-        float acc[16];
-        tmem_ld8x2(tl + (uint32_t)(dx * DW_NC + 8 * j), tl + (uint32_t)(dx * DW_NC + 8 * (DW_G + j)), acc);
-        const int dy = i - 1 - j;
-        if (dy >= -1 && dy <= 1) {
-          float4* d = reinterpret_cast<float4*>(red + (i * 3 + dy + 1) * 256 + ci * 16);
+  if (w >= 6 && sflag == 0) {
+    const int t = tid - 192;
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            d[c] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
-        }
-        __syncwarp();
-      }
+    for (int c = 0; c < 8; ++c)
+#pragma unroll
+      for (int o = 16; o > 1; o >>= 1) bacc[c] += __shfl_xor_sync(0xffffffffu, bacc[c], o);
+    if (lane < 2)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) bred[w - 6][8 * lane + c] = bacc[c];
+    asm volatile("bar.sync 2, 64;" ::: "memory");
+    if (t < 16) atomicAdd(a.db + t, bred[0][t] + bred[1][t]);
+  } else if (w >= 2 && sflag == 0) {
+    const int t = tid - 64;
+    const int i = 4 * (w & 1) + (lane >> 3), ci = 8 * ((w & 3) >> 1) + (lane & 7);
+    float* red = reinterpret_cast<float*>(smem);  // [i][dy + 1][ci][co]
+    auto put = [&](int d, const float v[16]) {
+      float4* o = reinterpret_cast<float4*>(red + (i * 3 + d) * 256 + ci * 16);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) o[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+    };
+    auto add_taps = [&](int dx) {
       asm volatile("bar.sync 1, 128;" ::: "memory");
       for (int e = t; e < 3 * 64; e += 128) {
         const int r = e >> 6, f = e & 63;  // dy + 1, float4 of the 16 x 16 block
@@ -1009,17 +1082,29 @@ __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
         atomicAdd(reinterpret_cast<float4*>(a.dW + (size_t)tap * CH * CH) + f, sum);
       }
       asm volatile("bar.sync 1, 128;" ::: "memory");
-    }
-    if (bias) {
+    };
+    if (one_chain) {
+      const int i0 = 4 * (w & 1);
+      const uint32_t tl = tmem + ((uint32_t)(32 * (w & 3)) << 16);
+#pragma unroll 1
+      for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll 1
+        for (int j = max(0, i0 - 2); j < min(DW_G, i0 + 4); ++j) {  // the same for the whole warp
+          float v[16];
+          tmem_ld8x2(tl + (uint32_t)(dx * DW_NC + 8 * j), tl + (uint32_t)(dx * DW_NC + 8 * (DW_G + j)), v);
+          if (i - j >= 0 && i - j < 3) put(i - j, v);
+          __syncwarp();
+        }
+        add_taps(dx);
+      }
+    } else {
 #pragma unroll
-      for (int c = 0; c < 8; ++c)
+      for (int dx = 0; dx < 3; ++dx) {
 #pragma unroll
-        for (int o = 16; o > 1; o >>= 1) bacc[c] += __shfl_xor_sync(0xffffffffu, bacc[c], o);
-      if (lane < 2)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) bred[w - 2][8 * lane + c] = bacc[c];
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (t < 16) atomicAdd(a.db + t, bred[0][t] + bred[1][t] + bred[2][t] + bred[3][t]);
+        for (int d = 0; d < 3; ++d)
+          if (i - d >= 0 && i - d < DW_G) put(d, acc[dx][d]);
+        add_taps(dx);
+      }
     }
   }
   tc_fence_before();
@@ -1062,6 +1147,7 @@ static sim_status launch_dw(const bf16* in, const bf16* dz, int n, int B, float*
   // one CTA per SM (all 512 TMEM columns), a third of them for each dz
   const int ctas = std::min(a.units, std::max(1, sms / 3));
   a.per_cta = cdiv(a.units, ctas);
+  a.chain = std::max(1, DW_CHAIN / cdiv(a.xs, 16));
   a.dW = dW;
   a.db = db;
   a.err = err;

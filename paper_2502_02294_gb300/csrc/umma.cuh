@@ -60,6 +60,17 @@ __device__ __forceinline__ void umma_bf16_acc(uint32_t leader, uint32_t d_tmem, 
       "r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc));
 }
 
+// the same with D = A B where acc is 0 (an accumulator's first MMA)
+__device__ __forceinline__ void umma_bf16(uint32_t leader, uint32_t d_tmem, uint32_t a_lo,
+                                          uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                          uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred e, p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 e, %0, 0;\n\t"
+      "setp.ne.b32 p, %7, 0;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%1], a, b, %6, p;\n\t}\n" ::"r"(leader),
+      "r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc));
+}
+
 // arrive once on the mbarrier when every tcgen05.mma issued so far by the elected lane is done
 __device__ __forceinline__ void umma_commit(uint32_t leader, uint64_t* mbar) {
   asm volatile(
@@ -67,6 +78,12 @@ __device__ __forceinline__ void umma_commit(uint32_t leader, uint64_t* mbar) {
       "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%1];\n\t}\n" ::"r"(leader),
       "r"(smem_u32(mbar))
       : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
+  uint64_t state;
+  asm volatile("mbarrier.arrive.shared::cta.b64 %0, [%1];" : "=l"(state) : "r"(smem_u32(mbar)) : "memory");
+  (void)state;
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
