@@ -29,9 +29,11 @@
  *     gives a message. Invalid arguments are rejected before any work is enqueued.
  *   - The library is not thread safe for one handle; distinct handles may be used from
  *     distinct threads.
- *   - Entries without a handle take their scratch memory in the order of `stream`; at most
- *     512 MB of it per device stays mapped between calls, until a handle is destroyed or an
- *     allocation of the library fails.
+ *   - Entries without a handle take their scratch memory in the order of `stream`. Once the host
+ *     has waited for the work (a stream, event or device synchronisation), at most 512 MB of it
+ *     per device stays mapped; calls queued without a wait keep their peak until then. What is kept
+ *     goes back to the system with sim_scratch_trim(), when a handle or closure is destroyed and
+ *     when an allocation of the library fails.
  */
 #ifndef DIFFHYDRO_H
 #define DIFFHYDRO_H
@@ -115,6 +117,10 @@ const char* sim_last_error(const sim_t* h);
 /* Number of CUDA kernels this library has launched in this process so far (all devices,
  * all threads; cuFFT's own kernels are not counted). Host-only, never fails. */
 int64_t sim_kernel_launches(void);
+
+/* Give the scratch memory that the entries without a handle keep on the current device back to
+ * the system (memory of calls still running stays). Never fails; the next call maps anew. */
+void sim_scratch_trim(void);
 
 /* ------------------------------------------------------------------ whole path */
 

@@ -13,4 +13,4 @@ from ._lib import (OBS_DENSITY, OBS_THERMAL)  # noqa: F401
 from .api import (Closure, Group, Simulation, SimRunFunction, refine_noise,  # noqa: F401
                   restrict_gas, restrict_particles, deposit_cic, gravity, gravity_adjoint,  # noqa: F401
                   interp_cic, philox, power_spectrum, simulate, subgrid, subgrid_adjoint,
-                  sweep, sweep_adjoint)
+                  scratch_trim, sweep, sweep_adjoint)

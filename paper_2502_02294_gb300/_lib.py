@@ -62,6 +62,7 @@ SIGNATURES = {
     "sim_params_default": (ctypes.c_int, [_PP]),
     "sim_last_error": (ctypes.c_char_p, [_P]),
     "sim_kernel_launches": (ctypes.c_int64, []),
+    "sim_scratch_trim": (None, []),
     "sim_init": (ctypes.c_int, [_PP, _P, _P, ctypes.POINTER(_P)]),
     "sim_init_batch": (ctypes.c_int, [_PP, _I32, _P, _P, ctypes.POINTER(_P)]),
     "sim_batch_size": (ctypes.c_int32, [_P]),

@@ -168,6 +168,12 @@ def cross_correlation(a, b, box: float, nbins: int):
     return k, rc, nm
 
 
+def scratch_trim():
+    """Give back the scratch memory that the single-call functions keep on the current device, for
+    another allocator in the process (sim_scratch_trim)."""
+    lib.sim_scratch_trim()
+
+
 def dot(a, b):
     """sum a_i b_i of two float32 device vectors, as a [1] float64 device tensor (sim_dot)."""
     _chk(b, F32, a.numel(), "b")

@@ -6,9 +6,10 @@
 // every call: three adjoint sweeps at 96^3 with a wait after them 594 -> 184 us (137-150 us
 // among other work), deposit + gravity + force at 128^3 591 -> 284 us, the spectra at 128^3
 // 664 -> 186 us. This pool keeps up to kKeep bytes mapped. Its allocations are ordered on the
-// caller's stream as before, so several threads and streams share it safely. What it keeps is
-// given back when a handle is destroyed, before cuFFT plans are made, and when an allocation of
-// this library fails. 512 MB is 0.2 % of the device and holds the largest scratch up to 188^3
+// caller's stream as before, so several threads and streams share it safely. The bound holds from
+// the next host synchronisation on (that is when CUDA applies a pool's threshold). What the pool
+// keeps is given back by sim_scratch_trim, when a handle is destroyed, before cuFFT plans are
+// made, and when an allocation of this library fails. 512 MB is 0.2 % of the device and holds the largest scratch up to 188^3
 // (20 n^3 floats, the x sweep's adjoint): above that the kernels take milliseconds and the
 // mapping matters less.
 #include <atomic>
@@ -89,3 +90,5 @@ void scratch_trim() {
 }
 
 }  // namespace dh
+
+extern "C" void sim_scratch_trim(void) { dh::scratch_trim(); }
