@@ -24,7 +24,9 @@
  *     as displacements s from the lattice site (x = q + s, periodic), momenta as p = a^2 dx/dt.
  *   - Units: length Mpc/h (comoving), velocity 100 km/s, time 1/H0 (so H0 = 1). Densities
  *     in units of the mean total matter density; the mean gas density is f_b = Omega_b/Omega_m.
- *     Gas variables: m = a rho U (U peculiar velocity), eps = a^2 rho (e + U^2/2).
+ *     Gas variables: m = a rho U (U peculiar velocity), eps = a^2 rho (e + U^2/2). In these units
+ *     densities are normal float32 numbers (1.2e-38 and more), and a sound speed below 1.1e-19
+ *     counts as zero.
  *   - Errors are returned as sim_status codes; nothing aborts or traps. sim_last_error()
  *     gives a message. Invalid arguments are rejected before any work is enqueued.
  *   - The library is not thread safe for one handle; distinct handles may be used from

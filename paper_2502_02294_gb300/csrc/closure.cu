@@ -14,14 +14,15 @@
 // padding positions stored beside it, so a run of lines of one half is one contiguous piece
 // and reaches shared memory as one bulk copy. The padding makes the operand of an in-plane
 // shift (dy, dx) the same tile moved by (dy P + dx) rows: descriptors only, no gather;
-// positions that fall on a padding column give discarded results. The three dz taps of one (dy, dx) form one N = 48 operand that updates three
-// output planes at once (see the geometry section).
+// positions that fall on a padding column give discarded results. The three dz taps of one
+// (dy, dx) form one N = 48 operand that updates three output planes at once (see the geometry
+// section).
 //
 // Backward: the gradient with respect to a layer's input is the same convolution with the
 // taps mirrored and each tap's matrix transposed (same kernel, other weight packing), its
 // epilogue multiplied by GELU' of the previous layer's pre-activation. The weight gradient
 // (a reduction over voxels of 27 rank-1 updates of 16 x 16) is a third tensor-core kernel:
-// M = (tap, input channel), N = output channel, K = voxels.
+// M = (input line, channel), N = (gradient line, channel), K = positions along x.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -725,7 +726,7 @@ static sim_status launch_conv(int mode, ConvArgs a, int B, cudaStream_t st) {
 // At the end the epilogue adds the six blocks of each tap through shared memory and the result to
 // dW with vector atomics. Two more warps sum db from the staged dz lines while the MMAs run, each of
 // the three dz CTAs (which stage the same lines) a third of the stages: all of it in one of them
-// made that one wait (shared-memory bandwidth; 102 us per 128^3 launch against 94).
+// made that one wait (102 us per 128^3 launch against 94).
 // Measured per layer, launches overlapped: 34 us at 64^3 x 2 and 73 us at 128^3 (33 and 80 with one
 // chain per CTA and db in the epilogue warps), against 303 us (64^3 x 2) for im2col tiles
 // transposed by stmatrix into K-major stages (N = 16), which spent its time on 27 loads and stores

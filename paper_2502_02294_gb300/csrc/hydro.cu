@@ -369,8 +369,11 @@ __device__ __forceinline__ void split_flux2(const float2 u[5], int f, float gam,
 // in a shared-memory ring (no shifted register windows, loads two cells ahead), no limiters in
 // the ramp-up and one-instruction reciprocals, a 128^3 sweep went from 29.3 M to 19.8 M warp
 // instructions and from 43 to 29 us under ncu (256^3: 275 -> 195 us in a run).
-template <int AXIS, int MINB>
-__global__ void __launch_bounds__(128, MINB)
+// Three resident blocks per SM (registers capped at 168, 12 warps per SM) measured fastest:
+// 25 us at 128^3 and 163 us at 256^3 per y or z sweep in a stream of sweeps, 34 us against 45
+// at four blocks (128 registers, spilling) in a 128^3 inference pass.
+template <int AXIS>
+__global__ void __launch_bounds__(128, 3)
 sweep_march2_kernel(const float* __restrict__ uin, float* __restrict__ uout, int n, SArg nua,
                     float gam, float eps, int L, const float* __restrict__ kick_g, SArg kick_K) {
   pdl_enter();
@@ -525,7 +528,9 @@ __device__ __forceinline__ void vanleer_vg2(float2 a, float2 b, float eps, float
 
 // split_flux with every rounding spelled out, for the marching adjoint's recomputation of the
 // forward stages: there the last bits decide which limiters are gated and the sign of a velocity
-// near zero, and which products the compiler contracts into FMAs depends on the code around.
+// near zero, and which products the compiler contracts into FMAs depends on the code around. So a
+// cell's adjoint does not depend on the segment length or the unrolling. (The forward sweeps round
+// in other places: a gate that the last bits decide can still differ from theirs.)
 // (The pressure enters the momentum flux and the enthalpy unrounded.)
 template <int F>
 __device__ __forceinline__ void split_flux_fixed(const float u[5], float gam, float FR[5],
@@ -1139,12 +1144,12 @@ sweep_adj_kernel(const float* __restrict__ uin, const float* __restrict__ lout,
 // paired march above n = 96 (n even; 25 us against 35 for the tile at 128^3, 56 against 72 at
 // 160^3, 163 against 280 at 256^3), the tile up to it (16.1 us against 16.7 at 96^3, 6.4
 // against 9.4 at 64^3: a march is one long dependent chain per thread, which small grids wait
-// for). Odd grids take the tile (280 us at 256 against 297 for the march on single lines). The adjoint defaults to the marching pair for every
-// axis: y/z directly (2.1x the tile at 256^3), x on x <-> y transposed copies (the x tile
-// takes ~320 us at 128^3 against ~170 us for a y/z pair), with segments fitted to whole
-// waves (at 128^3 three segments of 43 cells: every block resident at once, 140 us per
-// call in the benchmark pass against 156 us with 16-cell segments). sim_autotune times the
-// variants per handle.
+// for). Odd grids take the tile (280 us at 256 against 297 for the march on single lines).
+// The adjoint defaults to the march with fitted segments for every axis, y and z in one launch, x
+// in two on x <-> y transposed copies. Per call at 64^3 / 128^3 / 256^3: y / z 16 / 70 / 455 us (tile
+// 26 / 189 / 1475), x 22 / 111 / 828 us (tile 34 / 225 / 1770). Segments of 32 or 16 cells are within
+// 10 % at 128^3, of 32 cells 2 % faster at 256^3 and up to twice as long at 64^3. sim_autotune
+// times the variants per handle.
 static int pick_fwd(int axis, int n, int variant) {
   if (axis == 0) return SIM_SWEEP_TILE;
   if (variant != SIM_SWEEP_DEFAULT) return variant;
@@ -1246,25 +1251,15 @@ static sim_status launch_march_t(const float* uin, float* uout, int n, SArg nu, 
   return SIM_OK;
 }
 
-template <int AXIS, int MINB>
-static sim_status launch_march2_mb(const float* uin, float* uout, int n, SArg nu, float gam,
-                                   float eps, int B, cudaStream_t st, const float* kick_g,
-                                   SArg kick_K) {
-  const dim3 blk = line_block(n / 2, 128);
-  const int L = fit_segment(sweep_march2_kernel<AXIS, MINB>, n, B, kPairRamp, n / 2, blk, kPairSmem);
-  DH_CUDA_TRY((launch_pdl(sweep_march2_kernel<AXIS, MINB>, line_grid(n / 2, n, B, blk, cdiv(n, L)), blk, kPairSmem, st, uin, uout, n, nu, gam, eps, L, kick_g, kick_K)));
-  DH_LAUNCH_CHECK();
-  return SIM_OK;
-}
-
-// Three resident blocks per SM (registers capped at 168, 12 warps per SM) measured fastest:
-// 25 us at 128^3 and 163 us at 256^3 per y or z sweep in a stream of sweeps, 34 us against 45
-// at four blocks (128 registers, spilling) in a 128^3 inference pass.
 template <int AXIS>
 static sim_status launch_march2_t(const float* uin, float* uout, int n, SArg nu, float gam,
                                   float eps, int B, cudaStream_t st, const float* kick_g,
                                   SArg kick_K) {
-  return launch_march2_mb<AXIS, 3>(uin, uout, n, nu, gam, eps, B, st, kick_g, kick_K);
+  const dim3 blk = line_block(n / 2, 128);
+  const int L = fit_segment(sweep_march2_kernel<AXIS>, n, B, kPairRamp, n / 2, blk, kPairSmem);
+  DH_CUDA_TRY((launch_pdl(sweep_march2_kernel<AXIS>, line_grid(n / 2, n, B, blk, cdiv(n, L)), blk, kPairSmem, st, uin, uout, n, nu, gam, eps, L, kick_g, kick_K)));
+  DH_LAUNCH_CHECK();
+  return SIM_OK;
 }
 
 // the paired form needs two adjacent x columns per thread: y / z sweeps, n even
@@ -1452,7 +1447,7 @@ static sim_status set_sweep_attributes() {
   // the marching forms (x runs the adjoint of axis 1 on transposed copies)
   constexpr int A = AXIS == 0 ? 1 : AXIS, F = AXIS == 0 ? 1 : 1 + AXIS;
   DH_TRY(set_smem(sweep_adj_march_kernel<A, F, AXIS != 0>, kAdjSmem));
-  if (AXIS != 0) DH_TRY(set_smem(sweep_march2_kernel<A, 3>, kPairSmem));
+  if (AXIS != 0) DH_TRY(set_smem(sweep_march2_kernel<A>, kPairSmem));
   return SIM_OK;
 }
 

@@ -316,8 +316,8 @@ __global__ void __launch_bounds__(128, 16) deposit_kernel(const float* __restric
 // instance's pointers allow (add may alias out: each cell is read before it is written).
 // The accumulator is left as it is (clearing it here behind the read took 20 us per 128^3
 // against 7 us without): a simulation's is cleared for the next call by the Green's function
-// kernel, which is bound by its trigonometry and hides the stores, a single call's by a memset
-// before the deposit.
+// kernel (16 bytes per mode beside the 32 it moves; 8.3 us per 128^3 step, a launch fewer than a
+// memset), a single call's by a memset before the deposit.
 __global__ void fix_to_float_kernel(const unsigned long long* __restrict__ acc, SArg scale,
                                     const float* add, int add_stride, float offset, float* out,
                                     int N3) {
