@@ -57,10 +57,10 @@ SWEEP_BYTES_PER_CELL = 40      # sweep: 5 float32 fields read + 5 written
 SWEEP_ADJ_BYTES_PER_CELL = 60  # adjoint sweep: state and output adjoint read, input adjoint written
 # DRAM bytes per cell of one launch group (dram__bytes_read.sum + dram__bytes_write.sum) from
 # the ncu captures summarised in profiles/ (128^3, cold cache): forward sweep, the x tile
-# (43.2 MB) and the paired y / z forms (43.5, 44.2 MB) averaged; adjoint sweep (x, y, z average
+# (43.9 MB) and the paired y / z forms (43.5, 43.4 MB) averaged; adjoint sweep (x, y, z average
 # of the marching forms: x with its input transposes and a second pass, y / z in one pass)
-# (365.3 + 111.0 + 110.2) / 3 MB; None where no capture of the current kernel exists
-TRAFFIC_BYTES_PER_CELL = {"sweep": 20.82, "sweep_adjoint": 93.2}
+# (368.2 + 110.4 + 109.1) / 3 MB; None where no capture of the current kernel exists
+TRAFFIC_BYTES_PER_CELL = {"sweep": 20.79, "sweep_adjoint": 93.4}
 # the kernel forms (SWEEP_* per axis x, y, z) those captures measured
 PROFILED_VARIANTS = {"sweep": [1, 5, 5], "sweep_adjoint": [4, 4, 4]}
 # algorithmic bytes per cell of one timed launch group of each class (one particle per cell)
