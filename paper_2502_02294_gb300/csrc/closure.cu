@@ -799,6 +799,30 @@ __device__ __forceinline__ void tmem_ld8x2(uint32_t t0, uint32_t t1, float v[16]
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
+// the same for two pairs, both in flight before the wait
+__device__ __forceinline__ void tmem_ld8x4(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3,
+                                           float u[16], float v[16]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%32];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%33];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%34];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%35];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
+        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
+        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(t0), "r"(t1), "r"(t2), "r"(t3)
+      : "memory");
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    u[j] = __uint_as_float(r[j]);
+    v[j] = __uint_as_float(r[16 + j]);
+  }
+}
+
 __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ uint64_t full[DW_MAX_STAGES], empty[DW_MAX_STAGES], done;
@@ -1010,9 +1034,10 @@ __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
     }
   } else {
     // ---- epilogue: TMEM lane 8 (8 h + i) + c8 of warp w % 4 holds half h = (w % 4) / 2, input
-    //      lines i0 .. i0 + 3; columns 8 (6 h' + j) + c8'
-    const int i0 = 4 * (w & 1), il = lane >> 3;
-    const uint32_t tl = tmem + ((uint32_t)(32 * (w & 3)) << 16);
+    //      lines i0 .. i0 + 3; columns 8 (6 h' + j) + c8'. Four of the six dz lines meet them,
+    //      j0 .. j0 + 3
+    const int i0 = 4 * (w & 1), j0 = 2 * (w & 1), ij = i0 - j0 + (lane >> 3);
+    const uint32_t tl = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(8 * j0);
     bool ok = true;
     uint32_t use = 0, turn = 0;
     // (a CTA with one chain leaves it in TMEM)
@@ -1024,18 +1049,18 @@ __global__ void __launch_bounds__(DW_THREADS, 1) conv_dw_kernel(DwArgs a) {
       for (int dx = 0; dx < 3; ++dx) {
         const uint32_t slot = (use + dx) % DW_SLOTS, ts = tl + slot * DW_NC;
 #pragma unroll
-        for (int jj = 0; jj < 6; ++jj) {
-          const int j = i0 - 2 + jj;  // the same for the whole warp
-          if (j < 0 || j >= DW_G) continue;
-          float v[16];
-          tmem_ld8x2(ts + (uint32_t)(8 * j), ts + (uint32_t)(8 * (DW_G + j)), v);
+        for (int q = 0; q < 4; q += 2) {
+          float v[2][16];
+          tmem_ld8x4(ts + (uint32_t)(8 * q), ts + (uint32_t)(8 * (DW_G + q)), ts + (uint32_t)(8 * (q + 1)),
+                     ts + (uint32_t)(8 * (DW_G + q + 1)), v[0], v[1]);
+          // dz line j = j0 + q meets input line i = i0 + lane / 8 at dy + 1 = d = i - j
 #pragma unroll
-          for (int d = 0; d < 3; ++d) {
-            // dy + 1 = d is the input line j + d
-            if (il == jj + d - 2)
+          for (int d = 0; d < 3; ++d)
 #pragma unroll
-              for (int c = 0; c < 16; ++c) acc[dx][d][c] += v[c];
-          }
+            for (int e = 0; e < 2; ++e)
+              if (ij == d + q + e)
+#pragma unroll
+                for (int c = 0; c < 16; ++c) acc[dx][d][c] += v[e][c];
         }
         tc_fence_before();
         __syncwarp();
